@@ -255,7 +255,13 @@ lsp_status lsp_hj_solve(lsp_grid* grid, const lsp_solve_opts* opts, void* phi,
  * step count is odd), lsp_hj_step writes the stage field and copies it
  * back.  Every other stage on such a tile (RK1, RK3, lsp_hj_rate, the
  * adjoint's forward) runs the scalar body of the same tile.  lsp_autotune
- * does not try it.  A tile
+ * does not try it.
+ * pair = 6 (ENO2 and ENO3) is the register-marching ENO kernel: a thread
+ * owns 2 rows (in 4-D on 2 slabs of the slowest axis) at one node of the
+ * fastest axis, so a CTA has tb x ta/2 threads; tb is at most 64 and ta
+ * even, neither larger than its axis (the last tile of an axis is moved back
+ * to end at the edge).  Results as pairs 3 and 4, to FP32 rounding; minb is
+ * not used.  A tile
  * whose pair the scheme
  * has no variant for makes the step use the generic kernel.  With local
  * dissipation coefficients or the variational clip (opts->diss, varform),
@@ -263,9 +269,11 @@ lsp_status lsp_hj_solve(lsp_grid* grid, const lsp_solve_opts* opts, void* phi,
  * state only (every dynamics but QUADRATIC); other tiles run the scalar
  * body with the local coefficients and the clip.
  *  lsp_set_tile(g, 0, 0, 0, 0, 0)   default: WENO5 16 x 16, 3 CTAs/SM, pair 2,
- *                                   chunks for ~3 waves (even length); other
- *                                   schemes 32 x 8, 3 CTAs/SM, chunks for ~2
- *                                   waves
+ *                                   chunks for ~3 waves (even length); ENO2
+ *                                   and ENO3 with GLF and no clip from 2^14
+ *                                   nodes a pair 6 tile fitted to the grid;
+ *                                   otherwise 32 x 8, 3 CTAs/SM, chunks for
+ *                                   ~2 waves
  *  lsp_set_tile(g, -1, 0, 0, 0, 0)  always use the generic kernel
  *  lsp_set_tile(g, tb, ta, ch, minb, pair) explicit; LSP_EINVAL unless
  *        the launch has <= 65535 z-blocks, minb is 2, 3 or 4 and either
@@ -275,7 +283,9 @@ lsp_status lsp_hj_solve(lsp_grid* grid, const lsp_solve_opts* opts, void* phi,
  *        200 KB of shared memory, or pair is 5 on a 3-D grid with tb*ta <=
  *        256, the tile with a 4-cell halo fitting 4 values per thread and
  *        with a 2-cell halo 3 (checked for ENO2; a step whose scheme's
- *        halo does not fit runs the generic kernel).
+ *        halo does not fit runs the generic kernel), or pair is 6 with at
+ *        most 256 threads, the tile's frame (2 halo (tb + ta) values) in 2
+ *        values per thread and fewer than 2^30 nodes.
  * lsp_get_tile reports the tile a step with `opts` would use (all -1 when
  * the generic kernel runs). */
 lsp_status lsp_set_tile(lsp_grid* grid, int tb, int ta, int ch, int minb, int pair);
@@ -288,7 +298,8 @@ lsp_status lsp_get_tile(const lsp_grid* grid, const lsp_solve_opts* opts, int* t
  * stage alone is timed) for a set of tile shapes (7 fixed, 2 fitted to the
  * grid), chunk lengths, occupancy targets and kernel variants (WENO5: pair 0,
  * 1, 2; ENO2 and ENO3: pair 0, 1, plus the face-shared runs of pairs 3 and
- * 4 on 3 widths x 6 row counts x 7 chunk lengths), re-time the
+ * 4 on 3 widths x 6 row counts x 7 chunk lengths and the 12 tiles of pair 6
+ * with the lowest estimated cost), re-time the
  * six fastest over longer windows and keep the best in the grid handle
  * (reported through tb/ta/ch/minb/pair, which may be NULL).  Waits for the
  * GPU.  For grids without a tiled kernel it selects the generic one (all

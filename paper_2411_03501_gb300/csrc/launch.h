@@ -36,6 +36,12 @@ template <int R>
 cudaError_t launch_stage_run_r(int ndim, int scheme, int dyn, const StageArgs<float>& a,
                                const Tile& t, cudaStream_t s);
 bool run_tile_ok(int ndim, int scheme, int run, int tb, int ta);
+// Register-marching ENO2/ENO3 kernel (stage_march.cuh), Tile.pair = 6:
+// tb x ta nodes of the two fastest axes and ch planes per CTA.
+template <int NDIM>
+cudaError_t launch_stage_march(int scheme, int dyn, const StageArgs<float>& a, const Tile& t,
+                               cudaStream_t s);
+bool march_tile_ok(int ndim, int scheme, const Tile& t, const int* n);
 // The two stages of a TVD-RK2 step in one launch (stage_fused.cuh, Tile.pair
 // = 5): 3-D FP32 grids, GLF with state-only bounds; a.phi_s = phi^n, a.out =
 // phi^{n+1} (a different field), a.dt the step.

@@ -14,6 +14,7 @@
 #include "batched.h"
 #include "launch.h"
 #include "stage_generic.cuh"
+#include "stage_march.cuh"
 #include "stage_tiled.cuh"
 
 struct lsp_grid {
@@ -33,6 +34,9 @@ struct lsp_grid {
     // 1 = set explicitly (or by the autotuner), -1 = use the generic kernel
     int tile_mode = 0;
     lsp::Tile tile{0, 0, 0, 3, 0};
+    // default tiles of the register-marching ENO2 / ENO3 kernel (ch = 0: none
+    // fits), chosen once per grid (march_tiles)
+    lsp::Tile march[2] = {{0, 0, 0, 3, 6}, {0, 0, 0, 3, 6}};
 
     // cached CUDA graph of the last lsp_hj_solve with use_graph
     cudaGraphExec_t gexec = nullptr;
@@ -127,17 +131,88 @@ double cfl_dt_host(const lsp_grid* g, double cfl, double t, double t_final)
     return dt;
 }
 
-// Default tile: 32 x 8 threads over the two fastest axes, the march along
-// the third split into chunks so that at least ~2 waves of 2 CTAs per SM
-// are launched.
-// The tile used without lsp_set_tile / lsp_autotune: WENO5 runs the paired
+// Tiles of the register-marching ENO kernel (stage_march.cuh) for this grid,
+// cheapest first by the estimate
+//   (ch + 1) (CTAs per SM x warps per CTA + 16 x waves of resident CTAs),
+// in units of one warp's issue time per plane: a chunk costs about one plane
+// more than its length (its start), a plane costs each resident warp's
+// instructions plus about 16 warps' worth of latency per wave.  Fitted to
+// timed sweeps of TB, TA and ch on nine grids (300^3, 100^3, 57x43x211,
+// 250x41x60 ENO2; 45x160x120 and five 4-D grids ENO3): the first tile is
+// within 8 % of the best of the sweep on each.  Widths: the axis split evenly
+// into tiles of at most 64 nodes; rows: split evenly, or as many as fill 256
+// threads.
+void march_tiles(const lsp_grid* g, int scheme, std::vector<lsp::Tile>* out)
+{
+    out->clear();
+    const int d = g->ndim;
+    if (d != 3 && d != 4) return;
+    const int nB = g->n[d - 1], nA = g->n[d - 2], nS = g->n[d - 3];
+    const long long slabs = d == 4 ? (g->n[0] + 1) / 2 : 1;
+    std::vector<std::pair<double, lsp::Tile>> got;
+    const int k0 = (nB + lsp::kMarchMaxTB - 1) / lsp::kMarchMaxTB;
+    for (int k = k0; k <= k0 + 8; ++k) {
+        const int tb = (nB + k - 1) / k;
+        if (tb < 8 && k > k0) break;
+        const int most = std::min(lsp::kMarchThreads / tb, nA / lsp::kMarchRows);
+        for (int v = 0; v < 5; ++v) {
+            int nr = most;
+            if (v > 0) {
+                const int tiles = (nA + most * lsp::kMarchRows - 1) / (most * lsp::kMarchRows) + v - 1;
+                const int rows = (nA + tiles - 1) / tiles;
+                nr = std::min(most, (rows + lsp::kMarchRows - 1) / lsp::kMarchRows);
+            }
+            lsp::Tile t{tb, nr * lsp::kMarchRows, 1, 3, 6};
+            if (v > 0 && nr == most) continue;
+            const int threads = lsp::march_threads(t), warps = threads / 32;
+            const int resident = 65536 / ((d == 4 ? 128 : 80) * threads);
+            const long long plane_ctas = (long long)((nB + tb - 1) / tb) * ((nA + t.ta - 1) / t.ta) * slabs;
+            double best = INFINITY;
+            for (int sp = 1; sp <= nS; ++sp) {
+                const int ch = (nS + sp - 1) / sp;
+                if (sp > 1 && ch == (nS + sp - 2) / (sp - 1)) continue;  // as the last one
+                const long long ctas = plane_ctas * ((nS + ch - 1) / ch);
+                const long long per_sm = (ctas + lsp::sm_count() - 1) / lsp::sm_count();
+                const long long waves = (per_sm + resident - 1) / resident;
+                const double cost = (ch + 1.0) * ((double)per_sm * warps + 16.0 * waves);
+                lsp::Tile c = t;
+                c.ch = ch;
+                if (cost < best && lsp::tile_valid(d, scheme, c, g->n)) {
+                    best = cost;
+                    t.ch = ch;
+                }
+            }
+            if (best < INFINITY) got.push_back({best, t});
+        }
+    }
+    std::sort(got.begin(), got.end(), [](const std::pair<double, lsp::Tile>& x,
+                                         const std::pair<double, lsp::Tile>& y) { return x.first < y.first; });
+    for (const auto& c : got) out->push_back(c.second);
+}
+
+// Smaller grids keep the scalar kernel, whose body the batched solve runs for
+// these schemes, so that a small problem solved alone and in a batch gives
+// the same bits.  (Not the faster choice: rockets 21^3 4.3 us per stage with
+// the marching kernel against 8.8.)
+constexpr long long kMarchMinNodes = 1 << 14;
+
+// The tile used without lsp_set_tile / lsp_autotune.  WENO5 runs the paired
 // shared-face kernel on 16 x 16 tiles, chunked so that the launch has about
 // three waves of 3 CTAs per SM, with an even chunk length (the pairs of
-// planes); the other schemes the scalar kernel on 32 x 8 tiles, about two
+// planes).  ENO2/ENO3 with global coefficients run the register-marching
+// kernel (rockets 300^3: 165 us per stage against 388 for the scalar kernel's
+// 32 x 8 tiles, car4d 81^4: 438 against 860, 33 x 41 x 37 x 29: 21 against
+// 47); where no tile of it fits the grid, with local coefficients or the
+// clip, and for first order, the scalar kernel on 32 x 8 tiles, about two
 // waves of 2 CTAs per SM.
-lsp::Tile default_tile(const lsp_grid* g, int scheme)
+lsp::Tile default_tile(const lsp_grid* g, const lsp_solve_opts* o)
 {
-    const int d = g->ndim;
+    const int d = g->ndim, scheme = o->scheme;
+    if ((scheme == LSP_ENO2 || scheme == LSP_ENO3) && o->diss == LSP_DISS_GLF && !o->varform &&
+        g->npts >= kMarchMinNodes) {
+        const lsp::Tile& t = g->march[scheme == LSP_ENO3];
+        if (t.ch > 0) return t;
+    }
     const bool paired = scheme == LSP_WENO5;
     lsp::Tile t;
     t.tb = paired ? 16 : 32;
@@ -161,7 +236,7 @@ lsp::Tile tile_in_effect(const lsp_grid* g, const lsp_solve_opts* o)
 {
     lsp::Tile none{0, 0, 0, 0, 0};
     if (o->dtype != LSP_F32 || (g->ndim != 3 && g->ndim != 4) || g->tile_mode < 0) return none;
-    lsp::Tile t = g->tile_mode == 1 ? g->tile : default_tile(g, o->scheme);
+    lsp::Tile t = g->tile_mode == 1 ? g->tile : default_tile(g, o);
     return lsp::tile_valid(g->ndim, o->scheme, t, g->n) ? t : none;
 }
 
@@ -426,6 +501,11 @@ lsp_status lsp_grid_create(int ndim, const double* gmin, const double* gmax, con
         g->periodic[k] = bc[k] == LSP_BC_PERIODIC;
         g->dx[k] = g->periodic[k] ? (gmax[k] - gmin[k]) / (double)n[k]
                                   : (gmax[k] - gmin[k]) / (double)(n[k] - 1);
+    }
+    std::vector<lsp::Tile> tiles;
+    for (const int scheme : {LSP_ENO2, LSP_ENO3}) {
+        march_tiles(g, scheme, &tiles);
+        if (!tiles.empty()) g->march[scheme == LSP_ENO3] = tiles.front();
     }
     *out = g;
     return LSP_OK;
@@ -852,12 +932,17 @@ lsp_status lsp_autotune(lsp_grid* g, const lsp_solve_opts* o, const void* phi, v
     }
     const bool eno = o->scheme == LSP_ENO2 || o->scheme == LSP_ENO3;
     const int nrun = eno ? 3 * kRunRows : 0;
-    for (int si = 0; si < nshapes + nrun; ++si) {
-        const bool run = si >= nshapes;
+    // the register-marching kernel's cheapest tiles by its estimate
+    std::vector<lsp::Tile> marches;
+    if (eno) march_tiles(g, o->scheme, &marches);
+    const int nmarch = std::min((int)marches.size(), 12);
+    for (int si = 0; si < nshapes + nrun + nmarch; ++si) {
+        const bool march = si >= nshapes + nrun;
+        const bool run = si >= nshapes && !march;
         const int run_tb[3] = {16, 28, 32};
-        const int ri = (si - nshapes) % kRunRows;
-        const int sh[2] = {run ? run_tb[(si - nshapes) / kRunRows] : shapes[si][0],
-                           run ? run_rows[ri] : shapes[si][1]};
+        const int ri = run ? (si - nshapes) % kRunRows : 0;
+        const int sh[2] = {run ? run_tb[(si - nshapes) / kRunRows] : shapes[si < nshapes ? si : 0][0],
+                           run ? run_rows[ri] : shapes[si < nshapes ? si : 0][1]};
         if (run && ri >= 3) {
             bool dup = false;
             for (int q = 0; q < ri; ++q) dup |= run_rows[q] == sh[1];
@@ -875,6 +960,10 @@ lsp_status lsp_autotune(lsp_grid* g, const lsp_solve_opts* o, const void* phi, v
             if (pair == 1 && o->scheme == LSP_UPWIND1) continue;
             const int nS = g->n[d - 3];
             lsp::Tile t{sh[0], sh[1], (nS + sp - 1) / sp, run ? (pair == 3 ? 2 : 3) : minb, pair};
+            if (march) {
+                if (cand > 0) break;
+                t = marches[si - nshapes - nrun];
+            }
             if (!lsp::tile_valid(d, o->scheme, t, g->n)) continue;
             trial.tile = t;
             trial.tile_mode = 1;

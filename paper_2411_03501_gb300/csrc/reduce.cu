@@ -3,6 +3,7 @@
 // with partialFunc; alpha_k = max over the grid of the bound on |dH/dp_k|).
 #include "launch.h"
 #include "stage_generic.cuh"
+#include "stage_march.cuh"
 #include "stage_tiled.cuh"
 #include "adjoint.cuh"
 
@@ -33,6 +34,7 @@ bool tile_valid(int ndim, int scheme, const Tile& t, const int* n)
     if (t.minb < 2 || t.minb > 4) return false;
     const int nS = n[ndim - 3];
     const long long nz = (long long)((nS + t.ch - 1) / t.ch) * (ndim == 4 ? n[0] : 1);
+    if (t.pair == 6) return march_tile_ok(ndim, scheme, t, n);
     if (t.pair == 5) return fused_tile_ok(ndim, scheme, t, n);  // temporally blocked RK2
     if (t.pair == 3 || t.pair == 4) {  // face-shared ENO runs of 4 or 2 nodes
         return (scheme == ENO2 || scheme == ENO3) &&
@@ -47,6 +49,25 @@ bool tile_valid(int ndim, int scheme, const Tile& t, const int* n)
     // the tiled bodies; every shape the autotuner tries qualifies)
     if ((t.ta + 2 * G) * (t.tb + 2 * G) > 3 * t.ta * t.tb) return false;
     return nz <= 65535;
+}
+
+bool march_tile_ok(int ndim, int scheme, const Tile& t, const int* n)
+{
+    if (scheme != ENO2 && scheme != ENO3) return false;
+    const int G = ghost_width(scheme), ra = kMarchRows, r0 = march_slabs(ndim);
+    const int nB = n[ndim - 1], nA = n[ndim - 2], nS = n[ndim - 3];
+    // whole tiles inside the grid, whole blocks of rows
+    if (t.tb < 1 || t.tb > kMarchMaxTB || t.tb > nB || t.ta < ra || t.ta % ra || t.ta > nA) return false;
+    if (ndim == 4 && n[0] < r0) return false;
+    const int threads = march_threads(t);
+    if (threads > kMarchThreads) return false;
+    // the tile's frame in kMarchSlots values per thread
+    if (2 * G * (t.tb + t.ta) > kMarchSlots * threads) return false;
+    if (2 * sizeof(float) * r0 * (size_t)(t.ta + 2 * G) * kMarchPitch > kRunMaxSmem) return false;
+    long long npts = 1;  // 32-bit offsets inside a plane
+    for (int k = 0; k < ndim; ++k) npts *= n[k];
+    const long long nz = (long long)((nS + t.ch - 1) / t.ch) * (ndim == 4 ? (n[0] + r0 - 1) / r0 : 1);
+    return npts < (1LL << 30) && nz <= 65535 && (nA + t.ta - 1) / t.ta <= 65535;
 }
 
 bool run_tile_ok(int ndim, int scheme, int run, int tb, int ta)
@@ -65,9 +86,9 @@ cudaError_t launch_stage_tiled(int ndim, int scheme, int dyn, const StageArgs<fl
     // bodies, except on the WENO5 shared-face tile with state-only bounds,
     // whose kernel has a local variant
     if ((a.local_alpha || a.varform) && !(scheme == WENO5 && t.pair == 2 && dyn != QUADRATIC)) {
-        // the face-shared runs have no local variant: a one-node-per-thread
+        // the face-shared runs and marches have no local variant: a one-node-per-thread
         // tile of the same chunking runs the local body
-        const Tile tl = (t.pair == 3 || t.pair == 4) ? Tile{32, 8, t.ch, 3, 0}
+        const Tile tl = (t.pair == 3 || t.pair == 4 || t.pair == 6) ? Tile{32, 8, t.ch, 3, 0}
                                                      : Tile{t.tb, t.ta, t.ch, t.minb, 0};
         return launch_stage_tiled_local(ndim, scheme, dyn, a, tl, s);
     }
@@ -75,6 +96,9 @@ cudaError_t launch_stage_tiled(int ndim, int scheme, int dyn, const StageArgs<fl
         const Tile ts{t.tb, t.ta, t.ch, t.minb, 0};
         return launch_stage_tiled(ndim, scheme, dyn, a, ts, s);
     }
+    if (t.pair == 6)
+        return ndim == 3 ? launch_stage_march<3>(scheme, dyn, a, t, s)
+                         : launch_stage_march<4>(scheme, dyn, a, t, s);
     if (t.pair == 3) return launch_stage_run_r<4>(ndim, scheme, dyn, a, t, s);
     if (t.pair == 4) return launch_stage_run_r<2>(ndim, scheme, dyn, a, t, s);
     switch (t.minb) {

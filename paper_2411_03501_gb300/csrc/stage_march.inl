@@ -1,0 +1,62 @@
+// stage_march.inl -- instantiations and launcher of the register-marching
+// ENO2/ENO3 stage kernel (stage_march.cuh), Tile.pair = 6, for one
+// number of dimensions LSP_MARCH_NDIM (included by stage_march_3d.cu and
+// stage_march_4d.cu).
+#include "launch.h"
+#include "stage_march.cuh"
+
+namespace lsp {
+
+namespace {
+
+constexpr int ND = LSP_MARCH_NDIM;
+
+template <int SCHEME, int DYN>
+cudaError_t march_launch(const StageArgs<float>& a, const Tile& t, cudaStream_t s)
+{
+    constexpr int R0 = march_slabs(ND), G = ghost_width(SCHEME);
+    const int nB = a.n[ND - 1], nA = a.n[ND - 2], nS = a.n[ND - 3];
+    const int nchunks = (nS + t.ch - 1) / t.ch;
+    dim3 grid((nB + t.tb - 1) / t.tb, (nA + t.ta - 1) / t.ta,
+              nchunks * (ND == 4 ? (a.n[0] + R0 - 1) / R0 : 1));
+    const size_t smem = 2 * sizeof(float) * R0 * (t.ta + 2 * G) * kMarchPitch;
+    auto* fn = stage_march_kernel<ND, SCHEME, DYN, LSP_MARCH_MINB>;
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunMaxSmem);
+    if (attr != cudaSuccess) return attr;
+    fn<<<grid, march_threads(t), smem, s>>>(a, t.tb, t.ta, t.ch, nchunks);
+    return cudaGetLastError();
+}
+
+template <int SCHEME>
+cudaError_t march_dyn(int dyn, const StageArgs<float>& a, const Tile& t, cudaStream_t s)
+{
+    switch (dyn) {
+    case NORMAL_SPEED: return march_launch<SCHEME, NORMAL_SPEED>(a, t, s);
+    case TRANSLATE: return march_launch<SCHEME, TRANSLATE>(a, t, s);
+    case QUADRATIC: return march_launch<SCHEME, QUADRATIC>(a, t, s);
+    case AIR3D:
+        if constexpr (ND == 3) return march_launch<SCHEME, AIR3D>(a, t, s);
+        break;
+    case ROCKETS:
+        if constexpr (ND == 3) return march_launch<SCHEME, ROCKETS>(a, t, s);
+        break;
+    case CAR4D:
+        if constexpr (ND == 4) return march_launch<SCHEME, CAR4D>(a, t, s);
+        break;
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+template <>
+cudaError_t launch_stage_march<LSP_MARCH_NDIM>(int scheme, int dyn, const StageArgs<float>& a,
+                                               const Tile& t, cudaStream_t s)
+{
+    if (scheme == ENO2) return march_dyn<ENO2>(dyn, a, t, s);
+    if (scheme == ENO3) return march_dyn<ENO3>(dyn, a, t, s);
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace lsp
