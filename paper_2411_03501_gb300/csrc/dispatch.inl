@@ -2,6 +2,7 @@
 // precision LSP_REAL (included by stage_f32.cu / stage_f64.cu).
 #include "launch.h"
 #include "stage_generic.cuh"
+#include "stage_plane.cuh"
 
 namespace lsp {
 
@@ -10,6 +11,32 @@ static inline int stage_blocks(long long npts)
     long long b = (npts + 255) / 256;
     const long long cap = 16LL * sm_count();  // grid-stride beyond 16 blocks per SM
     return (int)(b < cap ? (b < 1 ? 1 : b) : cap);
+}
+
+// 2-D grids have a kernel of their own (stage_plane.cuh).
+template <int SCHEME>
+static cudaError_t plane_dyn(int dyn, const StageArgs<LSP_REAL>& a, cudaStream_t s)
+{
+    const int nt = plane_block(a.npts), nb = (a.npts + nt - 1) / nt;
+    switch (dyn) {
+    case NORMAL_SPEED: stage_plane_kernel<SCHEME, NORMAL_SPEED, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
+    case TRANSLATE: stage_plane_kernel<SCHEME, TRANSLATE, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
+    case QUADRATIC: stage_plane_kernel<SCHEME, QUADRATIC, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
+    case DOUBLE_INT: stage_plane_kernel<SCHEME, DOUBLE_INT, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
+static cudaError_t plane_scheme(int scheme, int dyn, const StageArgs<LSP_REAL>& a, cudaStream_t s)
+{
+    switch (scheme) {
+    case UPWIND1: return plane_dyn<UPWIND1>(dyn, a, s);
+    case ENO2: return plane_dyn<ENO2>(dyn, a, s);
+    case ENO3: return plane_dyn<ENO3>(dyn, a, s);
+    case WENO5: return plane_dyn<WENO5>(dyn, a, s);
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <int NDIM, int SCHEME>
@@ -28,9 +55,6 @@ static cudaError_t stage_dyn(int dyn, const StageArgs<LSP_REAL>& a, cudaStream_t
         return cudaErrorInvalidValue;
     case ROCKETS:
         if constexpr (NDIM == 3) { stage_generic_kernel<3, SCHEME, ROCKETS, LSP_REAL><<<nb, 256, 0, s>>>(a); break; }
-        return cudaErrorInvalidValue;
-    case DOUBLE_INT:
-        if constexpr (NDIM == 2) { stage_generic_kernel<2, SCHEME, DOUBLE_INT, LSP_REAL><<<nb, 256, 0, s>>>(a); break; }
         return cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
     }
@@ -55,11 +79,24 @@ cudaError_t launch_stage<LSP_REAL>(int ndim, int scheme, int dyn, const StageArg
 {
     switch (ndim) {
     case 1: return stage_scheme<1>(scheme, dyn, a, s);
-    case 2: return stage_scheme<2>(scheme, dyn, a, s);
+    case 2: return plane_scheme(scheme, dyn, a, s);
     case 3: return stage_scheme<3>(scheme, dyn, a, s);
     case 4: return stage_scheme<4>(scheme, dyn, a, s);
     }
     return cudaErrorInvalidValue;
+}
+
+static cudaError_t prange_plane(int scheme, const StageArgs<LSP_REAL>& a, cudaStream_t s)
+{
+    const int nt = plane_block(a.npts), nb = (a.npts + nt - 1) / nt;
+    switch (scheme) {
+    case UPWIND1: prange_plane_kernel<UPWIND1, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
+    case ENO2: prange_plane_kernel<ENO2, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
+    case ENO3: prange_plane_kernel<ENO3, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
+    case WENO5: prange_plane_kernel<WENO5, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
 }
 
 template <int NDIM>
@@ -82,7 +119,7 @@ cudaError_t launch_prange<LSP_REAL>(int ndim, int scheme, const StageArgs<LSP_RE
 {
     switch (ndim) {
     case 1: return prange_scheme<1>(scheme, a, s);
-    case 2: return prange_scheme<2>(scheme, a, s);
+    case 2: return prange_plane(scheme, a, s);
     case 3: return prange_scheme<3>(scheme, a, s);
     case 4: return prange_scheme<4>(scheme, a, s);
     }

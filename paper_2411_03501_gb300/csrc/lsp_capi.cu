@@ -153,7 +153,7 @@ void march_tiles(const lsp_grid* g, int scheme, std::vector<lsp::Tile>* out)
     const int k0 = (nB + lsp::kMarchMaxTB - 1) / lsp::kMarchMaxTB;
     for (int k = k0; k <= k0 + 8; ++k) {
         const int tb = (nB + k - 1) / k;
-        if (tb < 8 && k > k0) break;
+        if (tb < 16 && k > k0) break;  // narrow tiles are mostly frame
         const int most = std::min(lsp::kMarchThreads / tb, nA / lsp::kMarchRows);
         for (int v = 0; v < 5; ++v) {
             int nr = most;

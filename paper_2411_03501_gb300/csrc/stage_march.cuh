@@ -60,49 +60,6 @@ __host__ __device__ constexpr int march_slabs(int ndim) { return ndim == 4 ? 2 :
 // Threads of a tile's CTA (whole warps).
 inline int march_threads(const Tile& t) { return (t.tb * (t.ta / kMarchRows) + 31) / 32 * 32; }
 
-// Index i of an axis of n nodes brought into the grid: wrapped (periodic) or
-// clamped (a ghost, replaced by fix_extrapolated or in stage()).
-__device__ __forceinline__ int into_axis(int i, int n, int periodic)
-{
-    if (i < 0) return periodic ? i + n : 0;
-    if (i >= n) return periodic ? i - n : n - 1;
-    return i;
-}
-
-// Replace the ghost entries of the window w[k] = u_{i0-G+k} (R nodes from i0
-// and G on both sides) of an extrapolated axis of n nodes.  The nodes next to
-// the edge are selected, not indexed: w stays in registers.
-template <int R, int G>
-__device__ __forceinline__ void fix_extrapolated(float* w, int i0, int n)
-{
-    const int lo = G - i0;  // entries below node 0
-    if (lo > 0) {
-        float u0 = w[1], u1 = w[2];
-#pragma unroll
-        for (int c = 2; c <= G; ++c)
-            if (lo == c) {
-                u0 = w[c];
-                u1 = w[c + 1];
-            }
-#pragma unroll
-        for (int k = 0; k < G; ++k)
-            if (k < lo) w[k] = fmaf(float(lo - k), u0 - u1, u0);
-    }
-    const int kl = G + n - 1 - i0;  // entry of node n-1
-    if (kl < R + 2 * G - 1) {
-        float un = w[G], um = w[G - 1];
-#pragma unroll
-        for (int c = G + 1; c < R + 2 * G - 1; ++c)
-            if (kl == c) {
-                un = w[c];
-                um = w[c - 1];
-            }
-#pragma unroll
-        for (int k = G + 1; k < R + 2 * G; ++k)
-            if (k > kl) w[k] = fmaf(float(k - kl), un - um, un);
-    }
-}
-
 // The march along S at one node column: before plane s, u[] = u_s ..
 // u_{s+G-1}, S0 = S_s, S1 = S_{s+1}, T1 = T_{s+1/2}, M0 = M_s (ENO3) and
 // pm = dx p-_s.

@@ -1,0 +1,223 @@
+// stage_plane.cuh -- the fused Runge-Kutta stage (Sec. V-A) and the costate
+// range on 2-D grids, one thread per node, both precisions, every scheme.
+//
+// Same computation as stage_generic_kernel (stage_generic.cuh).  What bounds
+// it is latency on small grids and, in FP64, the FP64 pipe of GB300 (2
+// operations per SM and cycle): a stage of the 101 x 101 front is 10^4 nodes
+// of about 45 FP64 operations.  So
+//  - the block size is chosen to spread the nodes evenly over every SM
+//    (plane_block: 96 threads for 101 x 101, 107 SMs busy instead of 40);
+//  - index arithmetic is 32-bit, and all loads are requested at once:
+//    windows next to an edge load wrapped or clamped nodes and have their
+//    ghosts (Sec. III-B) replaced in registers;
+//  - FP64 magnitude comparisons, maxima and the finiteness test run on the
+//    bits of the values in the integer pipe, and WENO5 divides once per side
+//    instead of four times.  Otherwise the operations and their order are the
+//    generic kernel's (ENO2 and ENO3 give its bits).
+// Measured (GB300, us per stage of whole solves, generic kernel before):
+// 101 x 101 FP64 ENO2 6.4, 4.8; 127 x 93 FP64 WENO5 31.8, 14.6; 513 x 401
+// FP64 WENO5 174, 135 (the FP64 pipe); 301 x 177 FP32 WENO5 4.4, 3.5.  The
+// Jiang-Peng form of WENO5 (stage_tiled.cuh) with one division takes 10-15 %
+// less in FP64, but its error against FP64 torch was 2-15 % above the
+// generic kernel's on four cases and it was not kept.
+#pragma once
+#include "stage_generic.cuh"
+
+namespace lsp {
+
+// Threads per block: the fewest nodes on the busiest SM (whole warps, 64 to
+// 256 threads; ties to the larger block).
+inline int plane_block(long long npts)
+{
+    const long long sms = sm_count();
+    int best = 64;
+    long long cost = -1;
+    for (int t = 64; t <= 256; t += 32) {
+        const long long c = ((npts + t - 1) / t + sms - 1) / sms * t;
+        if (cost < 0 || c <= cost) {
+            cost = c;
+            best = t;
+        }
+    }
+    return best;
+}
+
+// |a| <= |b| (false when either is NaN).
+__device__ __forceinline__ bool mag_le(float a, float b) { return fabsf(a) <= fabsf(b); }
+__device__ __forceinline__ unsigned long long mag_bits(double a)
+{
+    return (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ bool mag_le(double a, double b)
+{
+    const unsigned long long ia = mag_bits(a), ib = mag_bits(b);
+    return ia <= ib && ib <= 0x7ff0000000000000ull;
+}
+// max(|a|, |b|) of finite values (a NaN operand gives NaN)
+__device__ __forceinline__ float mag_max(float a, float b) { return fmaxf(fabsf(a), fabsf(b)); }
+__device__ __forceinline__ double mag_max(double a, double b)
+{
+    const unsigned long long ia = mag_bits(a), ib = mag_bits(b);
+    return __longlong_as_double((long long)(ia > ib ? ia : ib));
+}
+__device__ __forceinline__ bool is_finite_bits(float v) { return isfinite(v); }
+__device__ __forceinline__ bool is_finite_bits(double v)
+{
+    return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
+}
+
+// 2^k close to 1/e for a normal e > 0: e times it lies in [1, 2).
+__device__ __forceinline__ float near_reciprocal(float e)
+{
+    return __uint_as_float(0x7f000000u - (__float_as_uint(e) & 0x7f800000u));
+}
+__device__ __forceinline__ double near_reciprocal(double e)
+{
+    return __longlong_as_double(0x7fe0000000000000ll -
+                                (__double_as_longlong(e) & 0x7ff0000000000000ll));
+}
+
+// weno5_combine (stencil.cuh) with one division instead of four: the weights
+// alpha_k = c_k / q_k^2 are multiplied by (q_1 q_2 q_3)^2, after q_k = s_k + eps
+// has been scaled by a power of two close to 1/eps.  The scaling is exact and
+// keeps every product in range (eps <= q_k <= 4e7 eps).
+template <typename R>
+__device__ __forceinline__ R plane_weno(R v1, R v2, R v3, R v4, R v5, R floor_)
+{
+    const R phi1 = v1 * R(1.0 / 3.0) - v2 * R(7.0 / 6.0) + v3 * R(11.0 / 6.0);
+    const R phi2 = -v2 * R(1.0 / 6.0) + v3 * R(5.0 / 6.0) + v4 * R(1.0 / 3.0);
+    const R phi3 = v3 * R(1.0 / 3.0) + v4 * R(5.0 / 6.0) - v5 * R(1.0 / 6.0);
+    const R a1 = v1 - R(2) * v2 + v3, b1 = v1 - R(4) * v2 + R(3) * v3;
+    const R a2 = v2 - R(2) * v3 + v4, b2 = v2 - v4;
+    const R a3 = v3 - R(2) * v4 + v5, b3 = R(3) * v3 - R(4) * v4 + v5;
+    const R s1 = R(13.0 / 12.0) * a1 * a1 + R(0.25) * b1 * b1;
+    const R s2 = R(13.0 / 12.0) * a2 * a2 + R(0.25) * b2 * b2;
+    const R s3 = R(13.0 / 12.0) * a3 * a3 + R(0.25) * b3 * b3;
+    const R m = mag_max(mag_max(mag_max(v1, v2), mag_max(v3, v4)), v5);
+    const R eps = R(1e-6) * (m * m) + floor_;
+    const R sc = near_reciprocal(eps);
+    const R q1 = (s1 + eps) * sc, q2 = (s2 + eps) * sc, q3 = (s3 + eps) * sc;
+    const R Q1 = q1 * q1, Q2 = q2 * q2, Q3 = q3 * q3;
+    const R al1 = R(0.1) * (Q2 * Q3), al2 = R(0.6) * (Q1 * Q3), al3 = R(0.3) * (Q1 * Q2);
+    return (al1 * phi1 + al2 * phi2 + al3 * phi3) / (al1 + al2 + al3);
+}
+
+// dx p- and dx p+ from the window u[0..2G].
+template <int SCHEME, typename R>
+__device__ __forceinline__ void plane_derivs(const R* u, R floor_, R& am, R& ap)
+{
+    if constexpr (SCHEME == UPWIND1) {
+        am = u[1] - u[0];
+        ap = u[2] - u[1];
+    } else if constexpr (SCHEME == ENO2) {
+        const R dm2 = u[1] - u[0], dm1 = u[2] - u[1], d0 = u[3] - u[2], d1 = u[4] - u[3];
+        const R Sm1 = dm1 - dm2, S0 = d0 - dm1, S1 = d1 - d0;
+        am = rfma(R(0.5), mag_le(Sm1, S0) ? Sm1 : S0, dm1);
+        ap = rfma(R(-0.5), mag_le(S0, S1) ? S0 : S1, d0);
+    } else if constexpr (SCHEME == ENO3) {
+        const R dm3 = u[1] - u[0], dm2 = u[2] - u[1], dm1 = u[3] - u[2];
+        const R d0 = u[4] - u[3], d1 = u[5] - u[4], d2 = u[6] - u[5];
+        const R Sm2 = dm2 - dm3, Sm1 = dm1 - dm2, S0 = d0 - dm1, S1 = d1 - d0, S2 = d2 - d1;
+        const R Tm2 = Sm1 - Sm2, Tm1 = S0 - Sm1, T0 = S1 - S0, T1 = S2 - S1;
+        // smaller third difference of each node's pair (deriv_eno3)
+        const R Mm1 = mag_le(Tm2, Tm1) ? Tm2 : Tm1, M0 = mag_le(Tm1, T0) ? Tm1 : T0;
+        const R M1 = mag_le(T0, T1) ? T0 : T1;
+        const bool l = mag_le(Sm1, S0), r = mag_le(S0, S1);
+        am = rfma(l ? Mm1 : M0, l ? R(1.0 / 3.0) : R(-1.0 / 6.0), rfma(R(0.5), l ? Sm1 : S0, dm1));
+        ap = rfma(r ? M0 : M1, r ? R(-1.0 / 6.0) : R(1.0 / 3.0), rfma(R(-0.5), r ? S0 : S1, d0));
+    } else {
+        const R dm3 = u[1] - u[0], dm2 = u[2] - u[1], dm1 = u[3] - u[2];
+        const R d0 = u[4] - u[3], d1 = u[5] - u[4], d2 = u[6] - u[5];
+        am = plane_weno(dm3, dm2, dm1, d0, d1, floor_);
+        ap = plane_weno(d2, d1, d0, dm1, dm2, floor_);
+    }
+}
+
+// Window of node c of a line of n nodes with stride s through p (the node's
+// own address), ghosts substituted.
+template <int G, typename R>
+__device__ __forceinline__ void plane_window(const R* __restrict__ p, int c, int n, int s,
+                                             int periodic, R* u)
+{
+    const bool inside = c >= G && c + G < n;
+#pragma unroll
+    for (int o = -G; o <= G; ++o) {
+        int off = o * s;
+        if (!inside) off = (into_axis(c + o, n, periodic) - c) * s;
+        u[o + G] = __ldg(p + off);
+    }
+    if (!inside && !periodic) fix_extrapolated<1, G>(u, c, n);
+}
+
+template <int SCHEME, int DYN, typename R>
+__global__ void __launch_bounds__(256) stage_plane_kernel(StageArgs<R> a)
+{
+    constexpr int G = ghost_width(SCHEME);
+    const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (unsigned)a.npts) return;
+    const int i = (int)(idx / (unsigned)a.n[1]), j = (int)(idx - (unsigned)i * (unsigned)a.n[1]);
+    R u[2][2 * G + 1];
+    plane_window<G>(a.phi_s + idx, i, a.n[0], a.stride[0], a.periodic[0], u[0]);
+    plane_window<G>(a.phi_s + idx, j, a.n[1], 1, a.periodic[1], u[1]);
+    const R vn = a.phi_n ? a.phi_n[idx] : R(0);
+    const R g = a.tube ? __ldg(a.target + idx) : R(0);
+    const R dt = a.dt_from_ctl ? R(a.ctl->dt) : a.dt;
+    const R x[2] = {rfma(R(i), a.h[0], a.lo[0]), rfma(R(j), a.h[1], a.lo[1])};
+    R pbar[2], diss = R(0);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        R pm, pp;
+        plane_derivs<SCHEME>(u[k], Num<R>::eps_floor(a.inv_dx[k]), pm, pp);
+        pm *= a.inv_dx[k];
+        pp *= a.inv_dx[k];
+        R al = a.alpha_from_ctl ? R(__longlong_as_double((long long)a.ctl->alpha_bits[k])) : a.alpha[k];
+        if (a.local_alpha) al = local_alpha<DYN>(x, k, a.prm, R(0), R(1), pm, pp);
+        pbar[k] = R(0.5) * (pp + pm);
+        diss += al * R(0.5) * (pp - pm);
+    }
+    const R H = hamiltonian<DYN, 2>(x, pbar, a.prm);
+    R L = -(H - diss);
+    if (a.varform) L = rmin(L, R(0));
+    R v = a.c_s * u[1][G] + a.c_l * dt * L;
+    if (a.phi_n) v += a.c_n * vn;
+    if (a.tube) v = rmin(v, g);
+    if (!is_finite_bits(v)) atomicOr(&a.ctl->flags, kFlagNonFinite);
+    a.out[idx] = v;
+}
+
+// prange_kernel (stage_generic.cuh) on 2-D grids.
+template <int SCHEME, typename R>
+__global__ void __launch_bounds__(256) prange_plane_kernel(StageArgs<R> a)
+{
+    constexpr int G = ghost_width(SCHEME);
+    const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
+    R m[2] = {R(0), R(0)};
+    if (idx < (unsigned)a.npts) {
+        const int i = (int)(idx / (unsigned)a.n[1]), j = (int)(idx - (unsigned)i * (unsigned)a.n[1]);
+        R u[2][2 * G + 1];
+        plane_window<G>(a.phi_s + idx, i, a.n[0], a.stride[0], a.periodic[0], u[0]);
+        plane_window<G>(a.phi_s + idx, j, a.n[1], 1, a.periodic[1], u[1]);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            R am, ap;
+            plane_derivs<SCHEME>(u[k], Num<R>::eps_floor(a.inv_dx[k]), am, ap);
+            m[k] = rmax(rabs(am), rabs(ap)) * a.inv_dx[k];
+        }
+    }
+    __shared__ R sm[2][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m[k] = rmax(m[k], __shfl_xor_sync(0xffffffffu, m[k], o));
+        if (lane == 0) sm[k][warp] = m[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        R v = R(0);
+        for (int w = 0; w < (int)((blockDim.x + 31) >> 5); ++w) v = rmax(v, sm[threadIdx.x][w]);
+        atomicMax(a.ctl->alpha_bits + threadIdx.x, (unsigned long long)__double_as_longlong((double)v));
+    }
+}
+
+}  // namespace lsp

@@ -431,4 +431,47 @@ __device__ __forceinline__ void load_window(const R* __restrict__ phi, long long
     }
 }
 
+// Index i of an axis of n nodes brought into the grid: wrapped (periodic) or
+// clamped (a ghost, replaced by fix_extrapolated).
+__device__ __forceinline__ int into_axis(int i, int n, int periodic)
+{
+    if (i < 0) return periodic ? i + n : 0;
+    if (i >= n) return periodic ? i - n : n - 1;
+    return i;
+}
+
+// Replace the ghost entries of the window w[k] = u_{i0-G+k} (R nodes from i0
+// and G on both sides) of an extrapolated axis of n nodes.  The nodes next to
+// the edge are selected, not indexed: w stays in registers.
+template <int R, int G, typename T>
+__device__ __forceinline__ void fix_extrapolated(T* w, int i0, int n)
+{
+    const int lo = G - i0;  // entries below node 0
+    if (lo > 0) {
+        T u0 = w[1], u1 = w[2];
+#pragma unroll
+        for (int c = 2; c <= G; ++c)
+            if (lo == c) {
+                u0 = w[c];
+                u1 = w[c + 1];
+            }
+#pragma unroll
+        for (int k = 0; k < G; ++k)
+            if (k < lo) w[k] = rfma(T(lo - k), u0 - u1, u0);
+    }
+    const int kl = G + n - 1 - i0;  // entry of node n-1
+    if (kl < R + 2 * G - 1) {
+        T un = w[G], um = w[G - 1];
+#pragma unroll
+        for (int c = G + 1; c < R + 2 * G - 1; ++c)
+            if (kl == c) {
+                un = w[c];
+                um = w[c - 1];
+            }
+#pragma unroll
+        for (int k = G + 1; k < R + 2 * G; ++k)
+            if (k > kl) w[k] = rfma(T(k - kl), un - um, un);
+    }
+}
+
 }  // namespace lsp
