@@ -86,28 +86,30 @@ cudaError_t launch_stage<LSP_REAL>(int ndim, int scheme, int dyn, const StageArg
     return cudaErrorInvalidValue;
 }
 
-static cudaError_t prange_plane(int scheme, const StageArgs<LSP_REAL>& a, cudaStream_t s)
+static cudaError_t prange_plane(int scheme, const StageArgs<LSP_REAL>& a, const StepChoice& ch,
+                                cudaStream_t s)
 {
     const int nt = plane_block(a.npts), nb = (a.npts + nt - 1) / nt;
     switch (scheme) {
-    case UPWIND1: prange_plane_kernel<UPWIND1, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
-    case ENO2: prange_plane_kernel<ENO2, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
-    case ENO3: prange_plane_kernel<ENO3, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
-    case WENO5: prange_plane_kernel<WENO5, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
+    case UPWIND1: prange_plane_kernel<UPWIND1, LSP_REAL><<<nb, nt, 0, s>>>(a, ch); break;
+    case ENO2: prange_plane_kernel<ENO2, LSP_REAL><<<nb, nt, 0, s>>>(a, ch); break;
+    case ENO3: prange_plane_kernel<ENO3, LSP_REAL><<<nb, nt, 0, s>>>(a, ch); break;
+    case WENO5: prange_plane_kernel<WENO5, LSP_REAL><<<nb, nt, 0, s>>>(a, ch); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
 
 template <int NDIM>
-static cudaError_t prange_scheme(int scheme, const StageArgs<LSP_REAL>& a, cudaStream_t s)
+static cudaError_t prange_scheme(int scheme, const StageArgs<LSP_REAL>& a, const StepChoice& ch,
+                                 cudaStream_t s)
 {
     const int nb = stage_blocks(a.npts);
     switch (scheme) {
-    case UPWIND1: prange_kernel<NDIM, UPWIND1, LSP_REAL><<<nb, 256, 0, s>>>(a); break;
-    case ENO2: prange_kernel<NDIM, ENO2, LSP_REAL><<<nb, 256, 0, s>>>(a); break;
-    case ENO3: prange_kernel<NDIM, ENO3, LSP_REAL><<<nb, 256, 0, s>>>(a); break;
-    case WENO5: prange_kernel<NDIM, WENO5, LSP_REAL><<<nb, 256, 0, s>>>(a); break;
+    case UPWIND1: prange_kernel<NDIM, UPWIND1, LSP_REAL><<<nb, 256, 0, s>>>(a, ch); break;
+    case ENO2: prange_kernel<NDIM, ENO2, LSP_REAL><<<nb, 256, 0, s>>>(a, ch); break;
+    case ENO3: prange_kernel<NDIM, ENO3, LSP_REAL><<<nb, 256, 0, s>>>(a, ch); break;
+    case WENO5: prange_kernel<NDIM, WENO5, LSP_REAL><<<nb, 256, 0, s>>>(a, ch); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -115,13 +117,13 @@ static cudaError_t prange_scheme(int scheme, const StageArgs<LSP_REAL>& a, cudaS
 
 template <>
 cudaError_t launch_prange<LSP_REAL>(int ndim, int scheme, const StageArgs<LSP_REAL>& a,
-                                    cudaStream_t s)
+                                    const StepChoice& ch, cudaStream_t s)
 {
     switch (ndim) {
-    case 1: return prange_scheme<1>(scheme, a, s);
-    case 2: return prange_plane(scheme, a, s);
-    case 3: return prange_scheme<3>(scheme, a, s);
-    case 4: return prange_scheme<4>(scheme, a, s);
+    case 1: return prange_scheme<1>(scheme, a, ch, s);
+    case 2: return prange_plane(scheme, a, ch, s);
+    case 3: return prange_scheme<3>(scheme, a, ch, s);
+    case 4: return prange_scheme<4>(scheme, a, ch, s);
     }
     return cudaErrorInvalidValue;
 }

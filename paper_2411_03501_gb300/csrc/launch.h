@@ -13,7 +13,8 @@ cudaError_t launch_stage(int ndim, int scheme, int dyn, const StageArgs<R>& a, c
 
 // Costate range reduction for H = |p|^2/2 (alpha from the current field).
 template <typename R>
-cudaError_t launch_prange(int ndim, int scheme, const StageArgs<R>& a, cudaStream_t s);
+cudaError_t launch_prange(int ndim, int scheme, const StageArgs<R>& a, const StepChoice& ch,
+                          cudaStream_t s);
 
 // State-only global-LF coefficients (FP64).
 cudaError_t launch_alpha_state(int dyn, const GridGeom& g, unsigned long long* out, cudaStream_t s);

@@ -36,11 +36,18 @@ struct Ctl {
     unsigned long long alpha_bits[LSP_MAXD];  // p-dependent GLF alpha (bits of
                                               // a non-negative double; atomicMax)
     double dt;                                // step chosen on the device
-    double t;                                 // time of the device loop
+    double t;                                 // time after that step
     unsigned int flags;                       // bit 0: non-finite value produced
+    unsigned int ticket;                      // blocks done of the costate-range launch
+    unsigned int stop_at;                     // steps of the solve once its last is chosen, else 0
     unsigned int pad0;
-    unsigned long long reserved[24];
+    unsigned long long acc[LSP_MAXD];         // costate maxima being collected
+    unsigned long long steps;                 // steps chosen on the device so far
+    double dt_min, dt_max;                    // over those steps
+    unsigned long long reserved[8];
 };
+// flags .. acc are zero at the start of every call that uses the block
+constexpr size_t kCtlResetBytes = 4 * sizeof(unsigned int) + LSP_MAXD * sizeof(unsigned long long);
 static_assert(sizeof(Ctl) <= 256, "control block must fit 256 bytes");
 constexpr size_t kCtlBytes = 256;
 constexpr unsigned int kFlagNonFinite = 1u;
@@ -71,6 +78,28 @@ struct StageArgs {
     int dt_from_ctl;     // 1: read dt from ctl->dt
     int local_alpha;     // 1: LLF/LLLF coefficients per node instead of alpha[]
     int varform;         // 1: variational form, rate clipped at zero
+    int step;            // with dt_from_ctl: index of the step in the solve
 };
+
+// What the costate-range launch does with the maxima (dynamics whose alpha
+// depends on the field): 0 alpha alone, 1 also choose the solve's next step,
+// 2 its first step.
+struct StepChoice {
+    int mode;
+    double cfl, t0, t_final, t_stop;
+    double dx[LSP_MAXD];
+};
+
+#ifdef __CUDACC__
+// Steps are enqueued ahead of the device's choice of dt: those past the last
+// one leave every field alone.
+template <typename R>
+__device__ __forceinline__ bool past_last_step(const StageArgs<R>& a)
+{
+    if (!a.dt_from_ctl) return false;
+    const unsigned stop = a.ctl->stop_at;
+    return stop != 0 && (unsigned)a.step >= stop;
+}
+#endif
 
 }  // namespace lsp

@@ -18,6 +18,7 @@ template <int NDIM, int SCHEME, int DYN, typename R>
 __global__ void __launch_bounds__(256) stage_generic_kernel(StageArgs<R> a)
 {
     constexpr int G = ghost_width(SCHEME);
+    if (past_last_step(a)) return;
     R alpha[NDIM];
 #pragma unroll
     for (int k = 0; k < NDIM; ++k)
@@ -107,12 +108,51 @@ __global__ void __launch_bounds__(256) alpha_state_kernel(GridGeom g, unsigned l
     }
 }
 
+// End of a costate-range launch, by the first warp of every block with the
+// block's maxima in lanes 0..NDIM-1 of m: the last block to arrive moves the
+// grid's maxima to ctl->alpha_bits (clearing the accumulators for the next
+// launch, which saves a memset each) and, asked to, chooses the step: the
+// operations of the host's CFL step in the same order, so the same steps.
+template <int NDIM>
+__device__ __forceinline__ void finish_prange(Ctl* c, double m, int step, const StepChoice& ch)
+{
+    const int lane = threadIdx.x;
+    if (lane < NDIM) atomicMax(c->acc + lane, (unsigned long long)__double_as_longlong(m));
+    __threadfence();
+    __syncwarp();
+    if (lane != 0 || atomicAdd(&c->ticket, 1u) != gridDim.x - 1) return;
+    __threadfence();
+    double alpha[NDIM];
+#pragma unroll
+    for (int k = 0; k < NDIM; ++k) {
+        const unsigned long long b = atomicExch(c->acc + k, 0ull);
+        c->alpha_bits[k] = b;
+        alpha[k] = __longlong_as_double((long long)b);
+    }
+    c->ticket = 0;
+    if (ch.mode == 0) return;
+    const bool first = ch.mode == 2;
+    const double t = first ? ch.t0 : c->t;
+    double sum = 0.0;
+#pragma unroll
+    for (int k = 0; k < NDIM; ++k) sum += alpha[k] / ch.dx[k];
+    double dt = sum > 0.0 ? ch.cfl / sum : ch.t_final - t;
+    if (ch.t_final - t < dt) dt = ch.t_final - t;
+    c->dt = dt;
+    c->t = t + dt;
+    c->steps = (unsigned long long)step + 1;
+    c->dt_min = first ? dt : fmin(c->dt_min, dt);
+    c->dt_max = first ? fmax(0.0, dt) : fmax(c->dt_max, dt);
+    if (!(t + dt < ch.t_stop)) c->stop_at = (unsigned)step + 1;
+}
+
 // Costate range for H = |p|^2/2: alpha_k = max over nodes of max(|p-_k|,
-// |p+_k|) of the current stage field, into ctl->alpha_bits (zeroed before).
+// |p+_k|) of the current stage field, into ctl->alpha_bits.
 template <int NDIM, int SCHEME, typename R>
-__global__ void __launch_bounds__(256) prange_kernel(StageArgs<R> a)
+__global__ void __launch_bounds__(256) prange_kernel(StageArgs<R> a, StepChoice ch)
 {
     constexpr int G = ghost_width(SCHEME);
+    if (past_last_step(a)) return;
     R m[NDIM];
 #pragma unroll
     for (int k = 0; k < NDIM; ++k) m[k] = R(0);
@@ -144,10 +184,11 @@ __global__ void __launch_bounds__(256) prange_kernel(StageArgs<R> a)
         if (lane == 0) sm[k][warp] = v;
     }
     __syncthreads();
-    if (threadIdx.x < NDIM) {
+    if (threadIdx.x < 32) {
         double v = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = fmax(v, sm[threadIdx.x][w]);
-        atomicMax(a.ctl->alpha_bits + threadIdx.x, (unsigned long long)__double_as_longlong(v));
+        if (threadIdx.x < NDIM)
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = fmax(v, sm[threadIdx.x][w]);
+        finish_prange<NDIM>(a.ctl, v, a.step, ch);
     }
 }
 

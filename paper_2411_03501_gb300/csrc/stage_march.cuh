@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
     constexpr int RA = kMarchRows, R0 = march_slabs(NDIM);
     constexpr int G = ghost_width(SCHEME), P = kMarchPitch, NS = kMarchSlots;
     constexpr int AS = NDIM - 3, AA = NDIM - 2, AB = NDIM - 1;
+    if (past_last_step(a)) return;
     extern __shared__ float march_smem[];  // [buffer][slab][TA + 2G][P]
     const int nB = a.n[AB], nA = a.n[AA], nS = a.n[AS];
     const int sA = a.stride[AA], sS = a.stride[AS];

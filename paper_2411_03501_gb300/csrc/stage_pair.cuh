@@ -330,6 +330,7 @@ __device__ __forceinline__ void tiled_pair_body(const StageArgs<float>& a, int T
 template <int NDIM, int DYN, int MINB, bool FACES, int SCHEME = WENO5, bool LOCAL = false>
 __global__ void __launch_bounds__(256, MINB) stage_pair_kernel(StageArgs<float> a, int ch, int nchunks)
 {
+    if (past_last_step(a)) return;
     extern __shared__ __align__(16) unsigned char smem_pair[];
     float* tile = reinterpret_cast<float*>(smem_pair);
     tiled_pair_body<NDIM, DYN, FACES, false, SCHEME, LOCAL>(a, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y,

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(256) stage_plane_kernel(StageArgs<R> a)
 {
     constexpr int G = ghost_width(SCHEME);
     const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (unsigned)a.npts) return;
+    if (idx >= (unsigned)a.npts || past_last_step(a)) return;
     const int i = (int)(idx / (unsigned)a.n[1]), j = (int)(idx - (unsigned)i * (unsigned)a.n[1]);
     R u[2][2 * G + 1];
     plane_window<G>(a.phi_s + idx, i, a.n[0], a.stride[0], a.periodic[0], u[0]);
@@ -187,9 +187,10 @@ __global__ void __launch_bounds__(256) stage_plane_kernel(StageArgs<R> a)
 
 // prange_kernel (stage_generic.cuh) on 2-D grids.
 template <int SCHEME, typename R>
-__global__ void __launch_bounds__(256) prange_plane_kernel(StageArgs<R> a)
+__global__ void __launch_bounds__(256) prange_plane_kernel(StageArgs<R> a, StepChoice ch)
 {
     constexpr int G = ghost_width(SCHEME);
+    if (past_last_step(a)) return;
     const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
     R m[2] = {R(0), R(0)};
     if (idx < (unsigned)a.npts) {
@@ -213,10 +214,11 @@ __global__ void __launch_bounds__(256) prange_plane_kernel(StageArgs<R> a)
         if (lane == 0) sm[k][warp] = m[k];
     }
     __syncthreads();
-    if (threadIdx.x < 2) {
+    if (threadIdx.x < 32) {
         R v = R(0);
-        for (int w = 0; w < (int)((blockDim.x + 31) >> 5); ++w) v = rmax(v, sm[threadIdx.x][w]);
-        atomicMax(a.ctl->alpha_bits + threadIdx.x, (unsigned long long)__double_as_longlong((double)v));
+        if (threadIdx.x < 2)
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = rmax(v, sm[threadIdx.x][w]);
+        finish_prange<2>(a.ctl, (double)v, a.step, ch);
     }
 }
 

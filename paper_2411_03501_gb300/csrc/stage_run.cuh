@@ -519,6 +519,7 @@ __device__ __forceinline__ void run_stage_body(const StageArgs<float>& a, int bx
 template <int NDIM, int SCHEME, int DYN, int R, int TBT, int MINB>
 __global__ void __launch_bounds__(256, MINB) stage_run_kernel(StageArgs<float> a, int ch, int nchunks)
 {
+    if (past_last_step(a)) return;
     extern __shared__ float4 run_smem[];
     run_stage_body<NDIM, SCHEME, DYN, R, TBT>(a, blockIdx.x, blockIdx.y, blockIdx.z % nchunks,
                                            blockIdx.z / nchunks, ch,

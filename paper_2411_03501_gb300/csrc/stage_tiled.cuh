@@ -352,6 +352,7 @@ __device__ __forceinline__ void tiled_stage_body(const StageArgs<R>& a, int TB, 
 template <int NDIM, int SCHEME, int DYN, typename R, int MINB, bool LOCAL = false>
 __global__ void __launch_bounds__(256, MINB) stage_tiled_kernel(StageArgs<R> a, int ch, int nchunks)
 {
+    if (past_last_step(a)) return;
     extern __shared__ unsigned char smem_raw[];
     R* tile = reinterpret_cast<R*>(smem_raw);
     tiled_stage_body<NDIM, SCHEME, DYN, R, false, LOCAL>(a, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y,
