@@ -712,7 +712,7 @@ def run_batched(args, rank: int, world: int, local_rank: int, emit: bool = True)
                    "parallelism": "problems split across ranks" if world > 1 else "single",
                    "l2": "flushed (512 MB write) between timed solves",
                    "launch": "persistent" if persistent else "stage-synchronous (graph)",
-                   "batch_chunk": args.batch_chunk or 128,
+                   "batch_chunk": args.batch_chunk or "auto",
                    "batch_tiles": {f"{d}-D": ["16x16", "32x8", "64x4"][(tiles >> (2 * (d - 2))) & 3]
                                    for d in (2, 3, 4)},
                    ("stage_synchronous_value" if persistent else "persistent_value"): alt_value,

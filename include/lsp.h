@@ -118,7 +118,8 @@ typedef struct {
                           lsp_hj_solve_batched captures its launches into
                           one graph and launches that                      */
     int batch_chunk;   /* batched solves: planes per CTA along the march of
-                          3-D/4-D problems (0 = 128)                        */
+                          3-D/4-D problems (0 = 4 to 128 by the work per
+                          resident CTA of one stage of the batch)         */
     int batch_persistent; /* batched solves: 1 = the whole solve as ONE
                           launch of resident CTAs that take (step, stage,
                           tile) items in order and wait on per-problem

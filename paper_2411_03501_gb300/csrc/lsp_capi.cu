@@ -1137,6 +1137,37 @@ size_t batch_persist_bytes(int nprob)
 // Test hook of the persistent batched launch (lsp_debug_stall_problem).
 int g_stall_problem = -1;
 
+// Planes per CTA when opts->batch_chunk is 0.  A stage of the whole batch has
+// x = (tiles x planes) / (3 CTAs x SMs) planes for each resident CTA: with
+// whole columns per CTA a small batch leaves most of them idle and waits for
+// the largest problem's column, with short chunks the persistent launch pays
+// its per-item overhead (counter, fences, dependency poll) and every CTA its
+// start more often.  Best of 4 .. 128 planes in milliseconds, against the
+// whole columns (128) used before, half 2-D fronts and half 3-D games, WENO5
+// RK3 (persistent; graph form in brackets):
+//   24 problems, x = 97: 32 planes 3.91, 128 5.06 (24: 4.04, 5.81)
+//   8 problems, x = 33: 16 planes 1.20, 2.69 (8: 1.25, 3.28)
+//   32 at half size, x = 21: 12 planes 0.92, 1.93 (8: 1.04, 2.30)
+//   4 at 0.4 size, x = 1: 4 planes 0.31, 1.06 (4: 0.34, 1.09)
+//   96 problems, x = 390: 128 planes 8.97 (32: 9.25, 64: 9.29, 128: 9.89)
+// which 5 + 0.31 x (persistent) and 4 + 0.2 x (graph) meet within 3 %.
+int batch_auto_chunk(int nprob, lsp_grid* const* grids, const lsp_solve_opts* o, int persistent)
+{
+    const bool local = o->diss != LSP_DISS_GLF || o->varform;
+    double planes = 0.0;
+    for (int i = 0; i < nprob; ++i) {
+        const lsp_grid* g = grids[i];
+        const int d = g->ndim;
+        int tb = 16, ta = 16;
+        lsp::batch_tile_dims(local ? 0 : (o->batch_tiles >> (2 * (d - 2))) & 3, &tb, &ta);
+        planes += (double)((g->n[d - 1] + tb - 1) / tb) * ((g->n[d - 2] + ta - 1) / ta) *
+                  (d >= 3 ? g->n[d - 3] : 1) * (d == 4 ? g->n[0] : 1);
+    }
+    const double x = planes / (3.0 * lsp::sm_count());
+    const double c = persistent ? 5.0 + 0.31 * x : 4.0 + 0.2 * x;
+    return c >= 128.0 ? 128 : std::max(4, (int)c / 2 * 2);
+}
+
 // Tile grid and field sizes of every problem; the total workspace bytes.
 // any_shape: size the block table for the largest tile count over every
 // shape (a workspace that serves any opts->batch_tiles).
@@ -1144,13 +1175,12 @@ void batch_geometry(int nprob, lsp_grid* const* grids, const lsp_solve_opts* o,
                     std::vector<BatchPlanEntry>& plan, size_t* bytes, long long* total_blocks,
                     bool any_shape = false)
 {
-    // 128 planes per CTA by default (a whole column of every problem up to
-    // 128 nodes along the march): the persistent launch's per-item overhead
-    // (counter, fences, dependency poll) is paid per tile, and the graph form
-    // gains too (256-problem workload: 67.5 / 67.0 G updates/s at 128 against
-    // 65.8 / 66.3 G at 64, 61.7 / 65.0 G at 32 and 54.3 / 61.5 G at 16,
-    // persistent / graph)
-    const int chunk = o->batch_chunk > 0 ? o->batch_chunk : 128;
+    const int chunk = o->batch_chunk > 0 ? o->batch_chunk
+                                         : batch_auto_chunk(nprob, grids, o, o->batch_persistent);
+    // a workspace sized for either form of the solve
+    const int finest = o->batch_chunk > 0 ? chunk
+                                          : std::min(batch_auto_chunk(nprob, grids, o, 0),
+                                                     batch_auto_chunk(nprob, grids, o, 1));
     plan.resize(nprob);
     size_t fields = 0;
     long long blocks = 0;
@@ -1177,7 +1207,8 @@ void batch_geometry(int nprob, lsp_grid* const* grids, const lsp_solve_opts* o,
                 nchunks = (nS + ch - 1) / ch;
             }
             const long long nb = (long long)nbx * nby * nchunks * (d == 4 ? g->n[0] : 1);
-            nb_max = std::max(nb_max, nb);
+            const int fine = d >= 3 ? (g->n[d - 3] + finest - 1) / finest : 1;
+            nb_max = std::max(nb_max, nb / nchunks * std::max(fine, nchunks));
             if (sh == shape) {
                 e.tb = tb;
                 e.ta = ta;
