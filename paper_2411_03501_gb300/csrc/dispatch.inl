@@ -19,13 +19,12 @@ static cudaError_t plane_dyn(int dyn, const StageArgs<LSP_REAL>& a, cudaStream_t
 {
     const int nt = plane_block(a.npts), nb = (a.npts + nt - 1) / nt;
     switch (dyn) {
-    case NORMAL_SPEED: stage_plane_kernel<SCHEME, NORMAL_SPEED, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
-    case TRANSLATE: stage_plane_kernel<SCHEME, TRANSLATE, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
-    case QUADRATIC: stage_plane_kernel<SCHEME, QUADRATIC, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
-    case DOUBLE_INT: stage_plane_kernel<SCHEME, DOUBLE_INT, LSP_REAL><<<nb, nt, 0, s>>>(a); break;
-    default: return cudaErrorInvalidValue;
+    case NORMAL_SPEED: return launch_dependent(stage_plane_kernel<SCHEME, NORMAL_SPEED, LSP_REAL>, nb, nt, 0, s, a);
+    case TRANSLATE: return launch_dependent(stage_plane_kernel<SCHEME, TRANSLATE, LSP_REAL>, nb, nt, 0, s, a);
+    case QUADRATIC: return launch_dependent(stage_plane_kernel<SCHEME, QUADRATIC, LSP_REAL>, nb, nt, 0, s, a);
+    case DOUBLE_INT: return launch_dependent(stage_plane_kernel<SCHEME, DOUBLE_INT, LSP_REAL>, nb, nt, 0, s, a);
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 static cudaError_t plane_scheme(int scheme, int dyn, const StageArgs<LSP_REAL>& a, cudaStream_t s)
@@ -91,13 +90,12 @@ static cudaError_t prange_plane(int scheme, const StageArgs<LSP_REAL>& a, const 
 {
     const int nt = plane_block(a.npts), nb = (a.npts + nt - 1) / nt;
     switch (scheme) {
-    case UPWIND1: prange_plane_kernel<UPWIND1, LSP_REAL><<<nb, nt, 0, s>>>(a, ch); break;
-    case ENO2: prange_plane_kernel<ENO2, LSP_REAL><<<nb, nt, 0, s>>>(a, ch); break;
-    case ENO3: prange_plane_kernel<ENO3, LSP_REAL><<<nb, nt, 0, s>>>(a, ch); break;
-    case WENO5: prange_plane_kernel<WENO5, LSP_REAL><<<nb, nt, 0, s>>>(a, ch); break;
-    default: return cudaErrorInvalidValue;
+    case UPWIND1: return launch_dependent(prange_plane_kernel<UPWIND1, LSP_REAL>, nb, nt, 0, s, a, ch);
+    case ENO2: return launch_dependent(prange_plane_kernel<ENO2, LSP_REAL>, nb, nt, 0, s, a, ch);
+    case ENO3: return launch_dependent(prange_plane_kernel<ENO3, LSP_REAL>, nb, nt, 0, s, a, ch);
+    case WENO5: return launch_dependent(prange_plane_kernel<WENO5, LSP_REAL>, nb, nt, 0, s, a, ch);
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 template <int NDIM>

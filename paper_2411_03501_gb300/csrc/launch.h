@@ -5,6 +5,26 @@
 
 namespace lsp {
 
+// Launch of a kernel that begins with stage_begin() (lsp_internal.h): its CTAs
+// may start while the previous kernel of the stream is still running, once
+// every CTA of that one has started.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                             A... args)
+{
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+
 struct GridGeom;
 
 // Fused stage (generic one-thread-per-node kernel).

@@ -132,7 +132,6 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
     constexpr int RA = kMarchRows, R0 = march_slabs(NDIM);
     constexpr int G = ghost_width(SCHEME), P = kMarchPitch, NS = kMarchSlots;
     constexpr int AS = NDIM - 3, AA = NDIM - 2, AB = NDIM - 1;
-    if (past_last_step(a)) return;
     extern __shared__ float march_smem[];  // [buffer][slab][TA + 2G][P]
     const int nB = a.n[AB], nA = a.n[AA], nS = a.n[AS];
     const int sA = a.stride[AA], sS = a.stride[AS];
@@ -209,17 +208,6 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
         f2[i] = 4u * (unsigned)p2;
     }
 
-    const float dt = a.dt_from_ctl ? float(a.ctl->dt) : a.dt;
-    const float cl = a.c_l * dt;
-    float hs[NDIM], ha[NDIM];  // 1/(2 dx_k) and alpha_k/(2 dx_k)
-#pragma unroll
-    for (int k = 0; k < NDIM; ++k) {
-        const float al = a.alpha_from_ctl
-                             ? float(__longlong_as_double((long long)a.ctl->alpha_bits[k]))
-                             : a.alpha[k];
-        hs[k] = 0.5f * a.inv_dx[k];
-        ha[k] = al * hs[k];
-    }
     // heading (axis 2): axis B in 3-D, axis A in 4-D
     constexpr bool kTrig = DYN == AIR3D || DYN == CAR4D || DYN == ROCKETS;
     constexpr int NT = NDIM == 4 ? RA : 1;
@@ -238,6 +226,20 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
     for (int r = 0; r < RA; ++r) st[r] = live && b >= bown && ar + r >= aown;
     const bool has_n = a.phi_n != nullptr, tube = a.tube != 0;
 
+    stage_wait();
+    stage_release();
+    if (past_last_step(a)) return;
+    const float dt = a.dt_from_ctl ? float(a.ctl->dt) : a.dt;
+    const float cl = a.c_l * dt;
+    float hs[NDIM], ha[NDIM];  // 1/(2 dx_k) and alpha_k/(2 dx_k)
+#pragma unroll
+    for (int k = 0; k < NDIM; ++k) {
+        const float al = a.alpha_from_ctl
+                             ? float(__longlong_as_double((long long)a.ctl->alpha_bits[k]))
+                             : a.alpha[k];
+        hs[k] = 0.5f * a.inv_dx[k];
+        ha[k] = al * hs[k];
+    }
     // plane of the lead value j (beyond the end of an extrapolated axis the
     // march continues its last difference instead)
     auto plane_of = [&](int j) { return a.phi_s + (size_t)(j < nS ? j : (perS ? j - nS : nS - 1)) * sS; };
@@ -249,8 +251,8 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
         for (int q = 0; q < R0; ++q)
 #pragma unroll
             for (int i = 0; i < NS; ++i) {
-                fv[q][i] = __ldg(at(plane, slab[G + q] + f1[i]));
-                gv[q][i] = ghosts ? __ldg(at(plane, slab[G + q] + f2[i])) : 0.0f;
+                fv[q][i] = *at(plane, slab[G + q] + f1[i]);
+                gv[q][i] = ghosts ? *at(plane, slab[G + q] + f2[i]) : 0.0f;
             }
     };
     // this thread's nodes and frame values into a buffer of the staged tile
@@ -277,9 +279,9 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
             float w[2 * G];
 #pragma unroll
             for (int k = 0; k < 2 * G; ++k)
-                w[k] = line_value<float>(at(a.phi_s, off), s_begin - G + k, nS, sS, perS);
+                w[k] = line_value<float, true>(at(a.phi_s, off), s_begin - G + k, nS, sS, perS);
             col_init<SCHEME>(w, m[q][r]);
-            lead[q][r] = __ldg(at(plane_of(s_begin + G), off));
+            lead[q][r] = *at(plane_of(s_begin + G), off);
         }
     stage(march_smem);
 
@@ -300,11 +302,11 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
 #pragma unroll
             for (int r = 0; r < RA; ++r) {
                 const unsigned off = slab[G + q] + own + r * rowb;
-                nlead[q][r] = __ldg(at(lplane, off));
+                nlead[q][r] = *at(lplane, off);
                 pn[q][r] = tg[q][r] = 0.0f;
                 if (st[r] && (NDIM < 4 || o0 + q >= oown)) {
                     if (has_n) pn[q][r] = *at(nplane, off);
-                    if (tube) tg[q][r] = __ldg(at(tplane, off));
+                    if (tube) tg[q][r] = *at(tplane, off);
                 }
             }
         float wo[NDIM == 4 ? 2 * G : 1][RA];
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
             for (int k = 0; k < 2 * G; ++k)
 #pragma unroll
                 for (int r = 0; r < RA; ++r)
-                    wo[k][r] = __ldg(at(plane, slab[k < G ? k : k + R0] + own + r * rowb));
+                    wo[k][r] = *at(plane, slab[k < G ? k : k + R0] + own + r * rowb);
         }
         if (more) frame(plane + sS);
         if (!perS && s + G >= nS) {  // beyond the end of an extrapolated axis

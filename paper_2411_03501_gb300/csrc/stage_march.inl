@@ -24,8 +24,7 @@ cudaError_t march_launch(const StageArgs<float>& a, const Tile& t, cudaStream_t 
     static const cudaError_t attr =
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunMaxSmem);
     if (attr != cudaSuccess) return attr;
-    fn<<<grid, march_threads(t), smem, s>>>(a, t.tb, t.ta, t.ch, nchunks);
-    return cudaGetLastError();
+    return launch_dependent(fn, grid, march_threads(t), smem, s, a, t.tb, t.ta, t.ch, nchunks);
 }
 
 template <int SCHEME>

@@ -314,7 +314,8 @@ __device__ __forceinline__ void tiled_pair_body(const StageArgs<float>& a, int T
             F2 v = fma2(cs, center, clk * L);
             if (a.phi_n)
                 v = fma2(cn, F2(ld_phin<COH>(a.phi_n + idx), second ? ld_phin<COH>(a.phi_n + idx + sS) : 0.f), v);
-            if (a.tube) v = min2(v, F2(__ldg(a.target + idx), second ? __ldg(a.target + idx + sS) : 0.f));
+            if (a.tube)
+                v = min2(v, F2(ld_in<COH>(a.target + idx), second ? ld_in<COH>(a.target + idx + sS) : 0.f));
             nonfinite |= !isfinite(v.x()) || (second && !isfinite(v.y()));
             a.out[idx] = v.x();
             if (second) a.out[idx + sS] = v.y();
@@ -330,10 +331,12 @@ __device__ __forceinline__ void tiled_pair_body(const StageArgs<float>& a, int T
 template <int NDIM, int DYN, int MINB, bool FACES, int SCHEME = WENO5, bool LOCAL = false>
 __global__ void __launch_bounds__(256, MINB) stage_pair_kernel(StageArgs<float> a, int ch, int nchunks)
 {
-    if (past_last_step(a)) return;
     extern __shared__ __align__(16) unsigned char smem_pair[];
     float* tile = reinterpret_cast<float*>(smem_pair);
-    tiled_pair_body<NDIM, DYN, FACES, false, SCHEME, LOCAL>(a, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y,
+    stage_wait();
+    stage_release();
+    if (past_last_step(a)) return;
+    tiled_pair_body<NDIM, DYN, FACES, true, SCHEME, LOCAL>(a, blockDim.x, blockDim.y, blockIdx.x, blockIdx.y,
                                blockIdx.z % nchunks, blockIdx.z / nchunks, ch, tile, threadIdx.x,
                                threadIdx.y);
 }

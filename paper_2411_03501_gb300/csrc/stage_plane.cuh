@@ -136,7 +136,7 @@ __device__ __forceinline__ void plane_derivs(const R* u, R floor_, R& am, R& ap)
 // Window of node c of a line of n nodes with stride s through p (the node's
 // own address), ghosts substituted.
 template <int G, typename R>
-__device__ __forceinline__ void plane_window(const R* __restrict__ p, int c, int n, int s,
+__device__ __forceinline__ void plane_window(const R* p, int c, int n, int s,
                                              int periodic, R* u)
 {
     const bool inside = c >= G && c + G < n;
@@ -144,7 +144,7 @@ __device__ __forceinline__ void plane_window(const R* __restrict__ p, int c, int
     for (int o = -G; o <= G; ++o) {
         int off = o * s;
         if (!inside) off = (into_axis(c + o, n, periodic) - c) * s;
-        u[o + G] = __ldg(p + off);
+        u[o + G] = p[off];
     }
     if (!inside && !periodic) fix_extrapolated<1, G>(u, c, n);
 }
@@ -154,13 +154,15 @@ __global__ void __launch_bounds__(256) stage_plane_kernel(StageArgs<R> a)
 {
     constexpr int G = ghost_width(SCHEME);
     const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (unsigned)a.npts || past_last_step(a)) return;
     const int i = (int)(idx / (unsigned)a.n[1]), j = (int)(idx - (unsigned)i * (unsigned)a.n[1]);
+    stage_wait();
+    stage_release();
+    if (idx >= (unsigned)a.npts || past_last_step(a)) return;
     R u[2][2 * G + 1];
     plane_window<G>(a.phi_s + idx, i, a.n[0], a.stride[0], a.periodic[0], u[0]);
     plane_window<G>(a.phi_s + idx, j, a.n[1], 1, a.periodic[1], u[1]);
     const R vn = a.phi_n ? a.phi_n[idx] : R(0);
-    const R g = a.tube ? __ldg(a.target + idx) : R(0);
+    const R g = a.tube ? a.target[idx] : R(0);
     const R dt = a.dt_from_ctl ? R(a.ctl->dt) : a.dt;
     const R x[2] = {rfma(R(i), a.h[0], a.lo[0]), rfma(R(j), a.h[1], a.lo[1])};
     R pbar[2], diss = R(0);
@@ -189,6 +191,8 @@ __global__ void __launch_bounds__(256) stage_plane_kernel(StageArgs<R> a)
 template <int SCHEME, typename R>
 __global__ void __launch_bounds__(256) prange_plane_kernel(StageArgs<R> a, StepChoice ch)
 {
+    stage_wait();
+    stage_release();
     constexpr int G = ghost_width(SCHEME);
     if (past_last_step(a)) return;
     const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;

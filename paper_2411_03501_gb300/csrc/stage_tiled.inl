@@ -25,21 +25,18 @@ static cudaError_t tiled_one(const StageArgs<float>& a, const Tile& t, cudaStrea
     if (local && !(kPairLocal && t.pair == 2)) return cudaErrorInvalidValue;
     if constexpr (SCHEME == WENO5 || SCHEME == ENO2 || SCHEME == ENO3) {
         if (t.pair == 1) {
-            stage_pair_kernel<NDIM, DYN, LSP_MINB, false, SCHEME><<<grid, block, 2 * smem, s>>>(a, t.ch, nchunks);
-            return cudaGetLastError();
+            return launch_dependent(stage_pair_kernel<NDIM, DYN, LSP_MINB, false, SCHEME>, grid, block, 2 * smem, s, a, t.ch, nchunks);
         }
     }
     if constexpr (SCHEME == WENO5) {
         if (t.pair == 2) {
             if constexpr (kPairLocal) {
                 if (local) {
-                    stage_pair_kernel<NDIM, DYN, LSP_MINB, true, WENO5, true>
-                        <<<grid, block, 2 * smem, s>>>(a, t.ch, nchunks);
-                    return cudaGetLastError();
+                    return launch_dependent(stage_pair_kernel<NDIM, DYN, LSP_MINB, true, WENO5, true>, grid, block, 2 * smem, s, a,
+                                            t.ch, nchunks);
                 }
             }
-            stage_pair_kernel<NDIM, DYN, LSP_MINB, true><<<grid, block, 2 * smem, s>>>(a, t.ch, nchunks);
-            return cudaGetLastError();
+            return launch_dependent(stage_pair_kernel<NDIM, DYN, LSP_MINB, true>, grid, block, 2 * smem, s, a, t.ch, nchunks);
         }
     }
     stage_tiled_kernel<NDIM, SCHEME, DYN, float, LSP_MINB><<<grid, block, smem, s>>>(a, t.ch, nchunks);
