@@ -261,8 +261,8 @@ lsp_status lsp_hj_solve(lsp_grid* grid, const lsp_solve_opts* opts, void* phi,
  * owns 2 rows (in 4-D on 2 slabs of the slowest axis) at one node of the
  * fastest axis, so a CTA has tb x ta/2 threads; tb is at most 64 and ta
  * even, neither larger than its axis (the last tile of an axis is moved back
- * to end at the edge).  Results as pairs 3 and 4, to FP32 rounding; minb is
- * not used.  A tile
+ * to end at the edge).  Results are those of pair 0 bit for bit; minb is not
+ * used.  A tile
  * whose pair the scheme
  * has no variant for makes the step use the generic kernel.  With local
  * dissipation coefficients or the variational clip (opts->diss, varform),
@@ -271,10 +271,9 @@ lsp_status lsp_hj_solve(lsp_grid* grid, const lsp_solve_opts* opts, void* phi,
  * body with the local coefficients and the clip.
  *  lsp_set_tile(g, 0, 0, 0, 0, 0)   default: WENO5 16 x 16, 3 CTAs/SM, pair 2,
  *                                   chunks for ~3 waves (even length); ENO2
- *                                   and ENO3 with GLF and no clip from 2^14
- *                                   nodes a pair 6 tile fitted to the grid;
- *                                   otherwise 32 x 8, 3 CTAs/SM, chunks for
- *                                   ~2 waves
+ *                                   and ENO3 with GLF and no clip a pair 6
+ *                                   tile fitted to the grid; otherwise 32 x 8,
+ *                                   3 CTAs/SM, chunks for ~2 waves
  *  lsp_set_tile(g, -1, 0, 0, 0, 0)  always use the generic kernel
  *  lsp_set_tile(g, tb, ta, ch, minb, pair) explicit; LSP_EINVAL unless
  *        the launch has <= 65535 z-blocks, minb is 2, 3 or 4 and either

@@ -131,14 +131,21 @@ double cfl_dt_host(const lsp_grid* g, double cfl, double t, double t_final)
     return dt;
 }
 
+// Longest chunk the marching kernel gets by default on 4-D grids, where longer
+// ones are slower than the estimate says (car4d 81^4, 41 x 12 tiles: 424 us
+// per stage with 21 planes, 434 with 27, 490 with 41, 485 with 81): the CTAs of
+// a wave drift apart and the slabs they share leave the caches.
+constexpr int kMarchMaxPlanes4 = 28;
+
 // Tiles of the register-marching ENO kernel (stage_march.cuh) for this grid,
 // cheapest first by the estimate
-//   (ch + 1) (CTAs per SM x warps per CTA + 16 x waves of resident CTAs),
+//   (ch + 1) (CTAs per SM x warps (1 + 0.05 frame / tile)
+//             + 16 x waves of resident CTAs),
 // in units of one warp's issue time per plane: a chunk costs about one plane
 // more than its length (its start), a plane costs each resident warp's
 // instructions plus about 16 warps' worth of latency per wave.  Fitted to
 // timed sweeps of TB, TA and ch on nine grids (300^3, 100^3, 57x43x211,
-// 250x41x60 ENO2; 45x160x120 and five 4-D grids ENO3): the first tile is
+// 250x41x60 ENO2; 45x160x120 and four 4-D grids ENO3): the first tile is
 // within 8 % of the best of the sweep on each.  Widths: the axis split evenly
 // into tiles of at most 64 nodes; rows: split evenly, or as many as fill 256
 // threads.
@@ -167,34 +174,31 @@ void march_tiles(const lsp_grid* g, int scheme, std::vector<lsp::Tile>* out)
             const int threads = lsp::march_threads(t), warps = threads / 32;
             const int resident = 65536 / ((d == 4 ? 128 : 80) * threads);
             const long long plane_ctas = (long long)((nB + tb - 1) / tb) * ((nA + t.ta - 1) / t.ta) * slabs;
+            if (!lsp::tile_valid(d, scheme, t, g->n)) continue;  // ch = 1: the most chunks
+            const double weight = warps * (1.0 + 0.05 * 2 * lsp::ghost_width(scheme) * (tb + t.ta) / (tb * t.ta));
             double best = INFINITY;
-            for (int sp = 1; sp <= nS; ++sp) {
+            int last = 0;
+            const int sp0 = d == 4 ? (nS + kMarchMaxPlanes4 - 1) / kMarchMaxPlanes4 : 1;
+            for (int sp = sp0; sp <= nS; sp += 1 + sp / 6) {
                 const int ch = (nS + sp - 1) / sp;
-                if (sp > 1 && ch == (nS + sp - 2) / (sp - 1)) continue;  // as the last one
+                if (ch == last) continue;
+                last = ch;
                 const long long ctas = plane_ctas * ((nS + ch - 1) / ch);
                 const long long per_sm = (ctas + lsp::sm_count() - 1) / lsp::sm_count();
                 const long long waves = (per_sm + resident - 1) / resident;
-                const double cost = (ch + 1.0) * ((double)per_sm * warps + 16.0 * waves);
-                lsp::Tile c = t;
-                c.ch = ch;
-                if (cost < best && lsp::tile_valid(d, scheme, c, g->n)) {
+                const double cost = (ch + 1.0) * (per_sm * weight + 16.0 * waves);
+                if (cost < best) {
                     best = cost;
                     t.ch = ch;
                 }
             }
-            if (best < INFINITY) got.push_back({best, t});
+            got.push_back({best, t});
         }
     }
-    std::sort(got.begin(), got.end(), [](const std::pair<double, lsp::Tile>& x,
+    std::stable_sort(got.begin(), got.end(), [](const std::pair<double, lsp::Tile>& x,
                                          const std::pair<double, lsp::Tile>& y) { return x.first < y.first; });
     for (const auto& c : got) out->push_back(c.second);
 }
-
-// Smaller grids keep the scalar kernel, whose body the batched solve runs for
-// these schemes, so that a small problem solved alone and in a batch gives
-// the same bits.  (Not the faster choice: rockets 21^3 4.3 us per stage with
-// the marching kernel against 8.8.)
-constexpr long long kMarchMinNodes = 1 << 14;
 
 // The tile used without lsp_set_tile / lsp_autotune.  WENO5 runs the paired
 // shared-face kernel on 16 x 16 tiles, chunked so that the launch has about
@@ -208,8 +212,7 @@ constexpr long long kMarchMinNodes = 1 << 14;
 lsp::Tile default_tile(const lsp_grid* g, const lsp_solve_opts* o)
 {
     const int d = g->ndim, scheme = o->scheme;
-    if ((scheme == LSP_ENO2 || scheme == LSP_ENO3) && o->diss == LSP_DISS_GLF && !o->varform &&
-        g->npts >= kMarchMinNodes) {
+    if ((scheme == LSP_ENO2 || scheme == LSP_ENO3) && o->diss == LSP_DISS_GLF && !o->varform) {
         const lsp::Tile& t = g->march[scheme == LSP_ENO3];
         if (t.ch > 0) return t;
     }
@@ -528,11 +531,6 @@ lsp_status lsp_grid_create(int ndim, const double* gmin, const double* gmax, con
         g->dx[k] = g->periodic[k] ? (gmax[k] - gmin[k]) / (double)n[k]
                                   : (gmax[k] - gmin[k]) / (double)(n[k] - 1);
     }
-    std::vector<lsp::Tile> tiles;
-    for (const int scheme : {LSP_ENO2, LSP_ENO3}) {
-        march_tiles(g, scheme, &tiles);
-        if (!tiles.empty()) g->march[scheme == LSP_ENO3] = tiles.front();
-    }
     *out = g;
     return LSP_OK;
 }
@@ -578,6 +576,13 @@ lsp_status lsp_set_dynamics(lsp_grid* g, int dyn, const double* params, int npar
     if (g->gexec) {
         cudaGraphExecDestroy(g->gexec);
         g->gexec = nullptr;
+    }
+    if (g->dyn < 0) {  // the grid's default tiles, once
+        std::vector<lsp::Tile> tiles;
+        for (const int scheme : {LSP_ENO2, LSP_ENO3}) {
+            march_tiles(g, scheme, &tiles);
+            if (!tiles.empty()) g->march[scheme == LSP_ENO3] = tiles.front();
+        }
     }
     for (int i = 0; i < LSP_NPARAM; ++i) g->prm[i] = i < need ? params[i] : 0.0;
     g->dyn = dyn;

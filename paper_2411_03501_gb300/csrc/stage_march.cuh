@@ -7,10 +7,8 @@
 // Hamiltonian with global-LF dissipation (Sec. IV-D), the RK combination and
 // the min with the target (Sec. VI-A); every ENO choice is made once per
 // cell face where both of its nodes belong to the thread (stencil.cuh).  The
-// results agree with the other bodies to FP32 rounding (1/dx is applied once
-// to the sum and once to the difference of a node's two derivatives; with
-// the scalar body's products and order of axes rockets 300^3 took 183 us per
-// stage instead of 160).
+// operations on a node, their order and the order of the axes are the scalar
+// body's, and so are the results, bit for bit.
 //
 // These schemes are bound by instruction issue on GB300, not by HBM, so the
 // layout is chosen to spend few instructions beside the arithmetic:
@@ -33,8 +31,8 @@
 //
 // Measured (GB300, us per stage of whole solves; default tile of the scalar
 // body before, its autotuned tile or run kernel in brackets, this kernel's
-// default tile now): rockets 300^3 ENO2 388 (182), 161; 100^3 22.3 (14.3),
-// 9.7; car4d 81^4 ENO3 860 (650), 438; 33 x 41 x 37 x 29 46.7, 21.1.  What
+// default tile now): rockets 300^3 ENO2 388 (182), 169; 100^3 20.8 (14.3),
+// 8.7; car4d 81^4 ENO3 870 (650), 438; 33 x 41 x 37 x 29 48, 21.5.  What
 // bounds it: instruction issue (51 % of the cycles, 150 instructions per node
 // in 3-D and 219 in 4-D, of which 45 and 125 are the scheme's arithmetic) and
 // the latency of the loads between barriers.
@@ -125,7 +123,9 @@ __device__ __forceinline__ void col_step(ColMarch<SCHEME>& m, float lead, float&
 // gridDim = (tiles along B, tiles along A, chunks x blocks of axis 0);
 // blockDim.x >= TB TA / RA threads, thread t at column t % TB of block
 // t / TB.  Offsets inside a plane are 32-bit: fields below 2^30 nodes.
-template <int NDIM, int SCHEME, int DYN, int MINB>
+// DEP: launched by launch_dependent (stage_wait, ordinary loads); otherwise an
+// ordinary launch reading the fields through the read-only path.
+template <int NDIM, int SCHEME, int DYN, int MINB, bool DEP>
 __global__ void __launch_bounds__(kMarchThreads, MINB)
     stage_march_kernel(StageArgs<float> a, int TB, int TA, int ch, int nchunks)
 {
@@ -168,6 +168,10 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
     const unsigned own = 4u * (unsigned)(ar * sA + b);
     auto at = [](const float* base, unsigned bytes) {
         return reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + bytes);
+    };
+    auto ld = [](const float* p) -> float {
+        if constexpr (DEP) return *p;
+        else return __ldg(p);
     };
 
     // This thread's share of the tile's frame: rows above and below (TB
@@ -226,20 +230,28 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
     for (int r = 0; r < RA; ++r) st[r] = live && b >= bown && ar + r >= aown;
     const bool has_n = a.phi_n != nullptr, tube = a.tube != 0;
 
-    stage_wait();
-    stage_release();
+    if constexpr (DEP) {
+        stage_wait();
+        stage_release();
+    }
     if (past_last_step(a)) return;
     const float dt = a.dt_from_ctl ? float(a.ctl->dt) : a.dt;
     const float cl = a.c_l * dt;
-    float hs[NDIM], ha[NDIM];  // 1/(2 dx_k) and alpha_k/(2 dx_k)
+    float ha[NDIM];  // alpha_k / 2
 #pragma unroll
-    for (int k = 0; k < NDIM; ++k) {
-        const float al = a.alpha_from_ctl
-                             ? float(__longlong_as_double((long long)a.ctl->alpha_bits[k]))
-                             : a.alpha[k];
-        hs[k] = 0.5f * a.inv_dx[k];
-        ha[k] = al * hs[k];
-    }
+    for (int k = 0; k < NDIM; ++k)
+        ha[k] = (a.alpha_from_ctl ? float(__longlong_as_double((long long)a.ctl->alpha_bits[k]))
+                                  : a.alpha[k]) *
+                0.5f;
+    // axis k's share of a node's costate and dissipation from dx p-, dx p+,
+    // rounded as the scalar body's (p+ + p-) / 2 and p+ - p- are compiled: the
+    // product of p- fused into the sum and the difference
+    auto axis = [&](int k, float am, float ap, float& pbar, float& diss) {
+        const float pp = __fmul_rn(ap, a.inv_dx[k]);
+        pbar = 0.5f * __fmaf_rn(am, a.inv_dx[k], pp);
+        diss = rfma(ha[k], __fmaf_rn(-am, a.inv_dx[k], pp), diss);
+    };
+
     // plane of the lead value j (beyond the end of an extrapolated axis the
     // march continues its last difference instead)
     auto plane_of = [&](int j) { return a.phi_s + (size_t)(j < nS ? j : (perS ? j - nS : nS - 1)) * sS; };
@@ -251,8 +263,8 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
         for (int q = 0; q < R0; ++q)
 #pragma unroll
             for (int i = 0; i < NS; ++i) {
-                fv[q][i] = *at(plane, slab[G + q] + f1[i]);
-                gv[q][i] = ghosts ? *at(plane, slab[G + q] + f2[i]) : 0.0f;
+                fv[q][i] = ld(at(plane, slab[G + q] + f1[i]));
+                gv[q][i] = ghosts ? ld(at(plane, slab[G + q] + f2[i])) : 0.0f;
             }
     };
     // this thread's nodes and frame values into a buffer of the staged tile
@@ -279,9 +291,9 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
             float w[2 * G];
 #pragma unroll
             for (int k = 0; k < 2 * G; ++k)
-                w[k] = line_value<float, true>(at(a.phi_s, off), s_begin - G + k, nS, sS, perS);
+                w[k] = line_value<float, DEP>(at(a.phi_s, off), s_begin - G + k, nS, sS, perS);
             col_init<SCHEME>(w, m[q][r]);
-            lead[q][r] = *at(plane_of(s_begin + G), off);
+            lead[q][r] = ld(at(plane_of(s_begin + G), off));
         }
     stage(march_smem);
 
@@ -302,11 +314,11 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
 #pragma unroll
             for (int r = 0; r < RA; ++r) {
                 const unsigned off = slab[G + q] + own + r * rowb;
-                nlead[q][r] = *at(lplane, off);
+                nlead[q][r] = ld(at(lplane, off));
                 pn[q][r] = tg[q][r] = 0.0f;
                 if (st[r] && (NDIM < 4 || o0 + q >= oown)) {
                     if (has_n) pn[q][r] = *at(nplane, off);
-                    if (tube) tg[q][r] = *at(tplane, off);
+                    if (tube) tg[q][r] = ld(at(tplane, off));
                 }
             }
         float wo[NDIM == 4 ? 2 * G : 1][RA];
@@ -315,15 +327,19 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
             for (int k = 0; k < 2 * G; ++k)
 #pragma unroll
                 for (int r = 0; r < RA; ++r)
-                    wo[k][r] = *at(plane, slab[k < G ? k : k + R0] + own + r * rowb);
+                    wo[k][r] = ld(at(plane, slab[k < G ? k : k + R0] + own + r * rowb));
         }
         if (more) frame(plane + sS);
         if (!perS && s + G >= nS) {  // beyond the end of an extrapolated axis
+            const float* last = a.phi_s + (size_t)(nS - 1) * sS;
 #pragma unroll
             for (int q = 0; q < R0; ++q)
 #pragma unroll
-                for (int r = 0; r < RA; ++r)
-                    lead[q][r] = m[q][r].u[G - 1] + (m[q][r].u[G - 1] - m[q][r].u[G - 2]);
+                for (int r = 0; r < RA; ++r) {
+                    const unsigned off = slab[G + q] + own + r * rowb;
+                    const float un = ld(at(last, off));
+                    lead[q][r] = fmaf(float(s + G - nS + 1), un - ld(at(last - sS, off)), un);
+                }
         }
 
         float pbar[R0][RA][NDIM], diss[R0][RA], center[R0][RA];
@@ -335,22 +351,9 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
                 center[q][r] = m[q][r].u[0];
                 float pm, pp;
                 col_step<SCHEME>(m[q][r], lead[q][r], pm, pp);
-                pbar[q][r][AS] = (pp + pm) * hs[AS];
-                diss[q][r] = ha[AS] * (pp - pm);
+                diss[q][r] = 0.0f;
+                axis(AS, pm, pp, pbar[q][r][AS], diss[q][r]);
                 lead[q][r] = nlead[q][r];
-            }
-        // axis B
-#pragma unroll
-        for (int q = 0; q < R0; ++q)
-#pragma unroll
-            for (int r = 0; r < RA; ++r) {
-                const float* p = cur + q * slab_floats + mine + r * P;
-                float w[2 * G + 1], pm, pp;
-#pragma unroll
-                for (int k = 0; k <= 2 * G; ++k) w[k] = k == G ? center[q][r] : p[k - G];
-                eno_line<SCHEME, 1>(w, &pm, &pp);
-                pbar[q][r][AB] = (pp + pm) * hs[AB];
-                diss[q][r] = fmaf(ha[AB], pp - pm, diss[q][r]);
             }
         // axis A
 #pragma unroll
@@ -362,11 +365,20 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
                 w[k] = k < G || k >= G + RA ? p[k * P] : center[q][(k - G) & (RA - 1)];
             eno_line<SCHEME, RA>(w, pm, pp);
 #pragma unroll
-            for (int r = 0; r < RA; ++r) {
-                pbar[q][r][AA] = (pp[r] + pm[r]) * hs[AA];
-                diss[q][r] = fmaf(ha[AA], pp[r] - pm[r], diss[q][r]);
-            }
+            for (int r = 0; r < RA; ++r) axis(AA, pm[r], pp[r], pbar[q][r][AA], diss[q][r]);
         }
+        // axis B
+#pragma unroll
+        for (int q = 0; q < R0; ++q)
+#pragma unroll
+            for (int r = 0; r < RA; ++r) {
+                const float* p = cur + q * slab_floats + mine + r * P;
+                float w[2 * G + 1], pm, pp;
+#pragma unroll
+                for (int k = 0; k <= 2 * G; ++k) w[k] = k == G ? center[q][r] : p[k - G];
+                eno_line<SCHEME, 1>(w, &pm, &pp);
+                axis(AB, pm, pp, pbar[q][r][AB], diss[q][r]);
+            }
         // axis 0
         if constexpr (NDIM == 4) {
 #pragma unroll
@@ -380,10 +392,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
                 if (edge0) fix_extrapolated<R0, G>(w, o0, a.n[0]);
                 eno_line<SCHEME, R0>(w, pm, pp);
 #pragma unroll
-                for (int q = 0; q < R0; ++q) {
-                    pbar[q][r][0] = (pp[q] + pm[q]) * hs[0];
-                    diss[q][r] = fmaf(ha[0], pp[q] - pm[q], diss[q][r]);
-                }
+                for (int q = 0; q < R0; ++q) axis(0, pm[q], pp[q], pbar[q][r][0], diss[q][r]);
             }
         }
         // Hamiltonian, rate, RK combination, tube
@@ -400,7 +409,7 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
                 x[AB] = xb;
                 constexpr int kT = NDIM == 4;
                 const float Hv = hamiltonian_sc<DYN, NDIM>(x, pbar[q][r], a.prm, sth[kT * r], cth[kT * r]);
-                const float L = diss[q][r] - Hv;
+                const float L = -(Hv - diss[q][r]);
                 float v = fmaf(cl, L, a.c_s * center[q][r]);
                 if (has_n) v = fmaf(a.c_n, pn[q][r], v);
                 if (tube) v = fminf(v, tg[q][r]);

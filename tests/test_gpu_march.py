@@ -1,5 +1,6 @@
 """The register-marching ENO2/ENO3 kernel (tile pair 6) against the FP64
-oracle at the edges of its tiles, and the tiles chosen by default."""
+oracle and, bit for bit, the scalar body at the edges of its tiles, and the
+tiles chosen by default."""
 import numpy as np
 import pytest
 import torch
@@ -42,11 +43,15 @@ def _check(spec, tile):
         P.set_tile(*tile, 3, 6)
         assert P.tile() == tile + (3, 6)
     assert P.tile()[4] == 6
+    S = B.Problem(spec)  # the scalar body: the same operations
+    S.set_tile(32, 8, 4, 3, 0)
     x = to_dev(phi, "f32")
-    out = torch.empty_like(x)
+    out, y = torch.empty_like(x), x.clone()
     P.rate(x, out)
     compare(out.double().cpu().numpy(), want, tol, flip_allowance(spec, phi, alpha), max_frac=0.05)
     P.step(x, to_dev(g, "f32"), t=0.0, dt=dt)
+    S.step(y, to_dev(g, "f32"), t=0.0, dt=dt)
+    assert torch.equal(x, y)
     got = x.double().cpu().numpy()
     compare(got, oracle.step(spec, phi, dt, 3, target=g), tol_step,
             step_flip_allowance(spec, phi, dt, 3, alpha, tol_step))
