@@ -269,8 +269,9 @@ lsp_status lsp_hj_solve(lsp_grid* grid, const lsp_solve_opts* opts, void* phi,
  * pair = 2 runs its local variant when the dynamics' bounds depend on the
  * state only (every dynamics but QUADRATIC); other tiles run the scalar
  * body with the local coefficients and the clip.
- *  lsp_set_tile(g, 0, 0, 0, 0, 0)   default: WENO5 16 x 16, 3 CTAs/SM, pair 2,
- *                                   chunks for ~3 waves (even length); ENO2
+ *  lsp_set_tile(g, 0, 0, 0, 0, 0)   default: WENO5 pair 2, 3 CTAs/SM, in 3-D a
+ *                                   tile and chunk fitted to the grid, in 4-D
+ *                                   16 x 16, chunks for ~3 waves; ENO2
  *                                   and ENO3 with GLF and no clip a pair 6
  *                                   tile fitted to the grid; otherwise 32 x 8,
  *                                   3 CTAs/SM, chunks for ~2 waves
