@@ -681,18 +681,13 @@ template <int DYN>
 __global__ void __launch_bounds__(256) alpha_argmax_kernel(GridGeom g, const double* alpha,
                                                           unsigned long long* out)
 {
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < g.npts;
-         idx += (long long)gridDim.x * blockDim.x) {
-        double x[LSP_MAXD] = {0.0, 0.0, 0.0, 0.0};
-        long long r = idx;
-        for (int k = g.ndim - 1; k >= 0; --k) {
-            x[k] = g.lo[k] + (double)(r % g.n[k]) * g.h[k];
-            r /= g.n[k];
-        }
-        for (int k = 0; k < g.ndim; ++k)
-            if (partial_bound<DYN>(x, k, g.prm) == alpha[k])
-                atomicMin(out + k, (unsigned long long)idx);
-    }
+#pragma unroll
+    for (int k = 0; k < LSP_MAXD; ++k)
+        if (k < g.ndim)
+            each_bound_node(g, bound_axes<DYN>(k), [&](long long idx, const double* x) {
+                if (partial_bound<DYN>(x, k, g.prm) == alpha[k])
+                    atomicMin(out + k, (unsigned long long)idx);
+            });
 }
 
 // ---------------------------------------------------------------------------

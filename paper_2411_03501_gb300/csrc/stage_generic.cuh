@@ -78,20 +78,44 @@ struct GridGeom {
     long long npts;
 };
 
+// Calls f(node index in C order, x) for this thread's share (grid-stride) of
+// the nodes with index 0 along every axis outside `axes`.
+template <typename F>
+__device__ __forceinline__ void each_bound_node(const GridGeom& g, unsigned axes, F f)
+{
+    long long count = 1, stride[LSP_MAXD] = {0, 0, 0, 0}, s = 1;
+    for (int k = g.ndim - 1; k >= 0; --k) {
+        stride[k] = s;
+        s *= g.n[k];
+        if ((axes >> k) & 1u) count *= g.n[k];
+    }
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
+         i += (long long)gridDim.x * blockDim.x) {
+        double x[LSP_MAXD] = {0.0, 0.0, 0.0, 0.0};
+        long long r = i, idx = 0;
+        for (int k = g.ndim - 1; k >= 0; --k) {
+            long long c = 0;
+            if ((axes >> k) & 1u) {
+                c = r % g.n[k];
+                r /= g.n[k];
+            }
+            x[k] = g.lo[k] + (double)c * g.h[k];
+            idx += c * stride[k];
+        }
+        f(idx, x);
+    }
+}
+
 template <int DYN>
 __global__ void __launch_bounds__(256) alpha_state_kernel(GridGeom g, unsigned long long* out)
 {
     double m[LSP_MAXD] = {0.0, 0.0, 0.0, 0.0};
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < g.npts;
-         idx += (long long)gridDim.x * blockDim.x) {
-        double x[LSP_MAXD] = {0.0, 0.0, 0.0, 0.0};
-        long long r = idx;
-        for (int k = g.ndim - 1; k >= 0; --k) {
-            x[k] = g.lo[k] + (double)(r % g.n[k]) * g.h[k];
-            r /= g.n[k];
-        }
-        for (int k = 0; k < g.ndim; ++k) m[k] = fmax(m[k], partial_bound<DYN>(x, k, g.prm));
-    }
+#pragma unroll
+    for (int k = 0; k < LSP_MAXD; ++k)
+        if (k < g.ndim)
+            each_bound_node(g, bound_axes<DYN>(k), [&](long long, const double* x) {
+                m[k] = fmax(m[k], partial_bound<DYN>(x, k, g.prm));
+            });
     __shared__ double sm[LSP_MAXD][8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int k = 0; k < g.ndim; ++k) {

@@ -401,6 +401,19 @@ __device__ __forceinline__ double partial_bound(const double* x, int k, const do
     }
 }
 
+// The axes whose coordinate partial_bound<DYN>(x, k, ..) depends on, as a bit
+// mask: the grid's maxima and the nodes attaining them are found on the nodes
+// of those axes alone (index 0 along the others).
+template <int DYN>
+__host__ __device__ constexpr unsigned bound_axes(int k)
+{
+    return DYN == AIR3D   ? (k == 0 ? 0b110u : k == 1 ? 0b101u : 0u)
+           : DYN == CAR4D ? (k <= 1 ? 0b1100u : 0u)
+           : DYN == ROCKETS ? (k <= 1 ? 0b101u : 0u)
+           : DYN == DOUBLE_INT ? (k == 0 ? 0b10u : 0u)
+                               : 0u;
+}
+
 // ---------------------------------------------------------------------------
 // Ghost-cell substitution for a window along one axis (Sec. III-B): the
 // value at axis coordinate j = i + o; periodic axes wrap, other axes
