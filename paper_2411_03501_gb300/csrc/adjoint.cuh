@@ -428,7 +428,7 @@ template <typename R>
 constexpr int adj_a_min_blocks() { return sizeof(R) == 4 ? 3 : 2; }
 
 template <int NDIM, int SCHEME, int DYN, typename R>
-__global__ void __launch_bounds__(256, adj_a_min_blocks<R>()) adj_stage_a(AdjArgs<R> a)
+__global__ void __launch_bounds__(256, adj_a_min_blocks<R>()) adj_stage_a(const __grid_constant__ AdjArgs<R> a)
 {
     constexpr int G = ghost_width(SCHEME);
     // per-thread partial sums in the field precision (a thread visits a few
@@ -466,12 +466,18 @@ __global__ void __launch_bounds__(256, adj_a_min_blocks<R>()) adj_stage_a(AdjArg
                 const int n = a.n[k], s = a.stride[k];
                 const float* ck =
                     reinterpret_cast<const float*>(a.gcontrib) + (long long)(7 * k + 3) * a.cstride + pidx;
-                const bool inner = pc[k] >= 3 && pc[k] < n - 3;
+                if (pc[k] >= 3 && pc[k] < n - 3) {  // no ghost cells: one stride
+                    const long long d = a.cstride - s;
+                    const float* q = ck - 3 * d;
+#pragma unroll
+                    for (int o = 0; o < 7; ++o, q += d) adj_cp4(sl + (2 + 7 * k + o) * 256, q);
+                    continue;
+                }
 #pragma unroll
                 for (int o = -3; o <= 3; ++o) {
                     float* dst = sl + (2 + 7 * k + o + 3) * 256;
                     int i = pc[k] - o;
-                    if (!inner && (i < 0 || i >= n)) {
+                    if (i < 0 || i >= n) {
                         if (!a.periodic[k]) {  // folded by the later stage's pass A
                             *dst = 0.0f;
                             continue;
@@ -534,33 +540,35 @@ __global__ void __launch_bounds__(256, adj_a_min_blocks<R>()) adj_stage_a(AdjArg
         // the window load, the derivative and the window gradient in the
         // code instead of NDIM: the unrolled form was bound by instruction
         // fetch); per-axis values go in and out of the small arrays by
-        // selects over compile-time indices, so they stay in registers.
+        // selects over compile-time indices, so they stay in registers; the
+        // launch's per-axis constants are indexed where they are
+        // (__grid_constant__: no copy, one constant load each).
         R x[NDIM], pm[NDIM], pp[NDIM], pbar[NDIM];
         R diss = R(0);
         // the stencil window of axis k at this node (ghost cells substituted)
         auto window = [&](int k, R* u) {
-            const int nk = pick<NDIM>(a.n, k), ck = pick<NDIM>(c, k);
-            const int sk = pick<NDIM>(a.stride, k);
+            const int nk = a.n[k], ck = pick<NDIM>(c, k);
+            const int sk = a.stride[k];
             if (ck >= 3 && ck < nk - 3) {  // no ghost cells in the window
                 const R* p0 = a.u + idx;
 #pragma unroll
                 for (int o = -3; o <= 3; ++o) u[o + 3] = __ldg(p0 + (long long)o * sk);
             } else {
-                load_window<R, 3>(a.u, idx, ck, nk, sk, pick<NDIM>(a.periodic, k), u);
+                load_window<R, 3>(a.u, idx, ck, nk, sk, a.periodic[k], u);
             }
         };
 #pragma unroll 1
         for (int k = 0; k < NDIM; ++k) {
             R u[7];
             window(k, u);
-            const R idk = pick<NDIM>(a.inv_dx, k);
+            const R idk = a.inv_dx[k];
             R pmk, ppk;
             deriv_fast<SCHEME>(u + (3 - G), idk, weno_floor12(idk), pmk, ppk);
             put<NDIM>(pm, k, pmk);
             put<NDIM>(pp, k, ppk);
             put<NDIM>(pbar, k, R(0.5) * (ppk + pmk));
-            diss += pick<NDIM>(a.alpha, k) * R(0.5) * (ppk - pmk);
-            put<NDIM>(x, k, pick<NDIM>(a.lo, k) + R(pick<NDIM>(c, k)) * pick<NDIM>(a.h, k));
+            diss += a.alpha[k] * R(0.5) * (ppk - pmk);
+            put<NDIM>(x, k, a.lo[k] + R(pick<NDIM>(c, k)) * a.h[k]);
         }
         R sth = R(0), cth = R(1);
         if constexpr (DYN == AIR3D || DYN == CAR4D || DYN == ROCKETS) rsincos(x[2], &sth, &cth);
@@ -589,14 +597,14 @@ __global__ void __launch_bounds__(256, adj_a_min_blocks<R>()) adj_stage_a(AdjArg
                       pick<NDIM>(acc_a, k) + w * R(0.5) * (pick<NDIM>(pp, k) - pick<NDIM>(pm, k)));
             R u[7], gm[7], gp[7];
             window(k, u);  // again: cheaper than holding NDIM windows in registers
-            const R idk = pick<NDIM>(a.inv_dx, k), alk = pick<NDIM>(a.alpha, k);
+            const R idk = a.inv_dx[k], alk = a.alpha[k];
             window_grad<SCHEME>(u, idk, weno_floor12(idk), gm, gp);
             const R hpk = pick<NDIM>(hp, k);
             const R sp = w * (R(-0.5) * hpk + R(0.5) * alk);
             const R sm = w * (R(-0.5) * hpk - R(0.5) * alk);
             R* out = a.contrib + (long long)(7 * k + 3) * a.cstride + idx;  // offset 0
-            const int n = pick<NDIM>(a.n, k), s = pick<NDIM>(a.stride, k), ck = pick<NDIM>(c, k);
-            const int perk = pick<NDIM>(a.periodic, k);
+            const int n = a.n[k], s = a.stride[k], ck = pick<NDIM>(c, k);
+            const int perk = a.periodic[k];
             if (perk || (ck >= 3 && ck < n - 3)) {  // no ghost position to fold
 #pragma unroll
                 for (int o = -3; o <= 3; ++o)
