@@ -134,7 +134,8 @@ def launch_accounting(spec, tile, stats) -> tuple[int, float, float, bool]:
 
 
 KERNEL_SOURCES = ["stencil.cuh", "stage_tiled.cuh", "stage_tiled.inl", "stage_generic.cuh",
-                  "pair2.cuh", "stage_pair.cuh", "stage_run.cuh", "stage_run.inl"]
+                  "pair2.cuh", "stage_pair.cuh", "stage_run.cuh", "stage_run.inl",
+                  "stage_march.cuh", "stage_march.inl"]
 
 
 def kernel_hash() -> str:

@@ -157,6 +157,7 @@ void march_tiles(const lsp_grid* g, int scheme, std::vector<lsp::Tile>* out)
     const int d = g->ndim;
     if (d != 3 && d != 4) return;
     const int nB = g->n[d - 1], nA = g->n[d - 2], nS = g->n[d - 3];
+    const long long sms = lsp::sm_count();
     const long long slabs = d == 4 ? (g->n[0] + 1) / 2 : 1;
     std::vector<std::pair<double, lsp::Tile>> got;
     const int k0 = (nB + lsp::kMarchMaxTB - 1) / lsp::kMarchMaxTB;
@@ -186,7 +187,7 @@ void march_tiles(const lsp_grid* g, int scheme, std::vector<lsp::Tile>* out)
                 if (ch == last) continue;
                 last = ch;
                 const long long ctas = plane_ctas * ((nS + ch - 1) / ch);
-                const long long per_sm = (ctas + lsp::sm_count() - 1) / lsp::sm_count();
+                const long long per_sm = (ctas + sms - 1) / sms;
                 const long long waves = (per_sm + resident - 1) / resident;
                 const double cost = (ch + 1.0) * (per_sm * weight + 16.0 * waves);
                 if (cost < best) {
@@ -217,6 +218,7 @@ lsp::Tile pair_tile(const lsp_grid* g)
     lsp::Tile best{0, 0, 0, 3, 2};
     if (g->ndim != 3) return best;
     const int nS = g->n[0], nA = g->n[1], nB = g->n[2], G = 3;
+    const long long sms = lsp::sm_count();
     double best_cost = INFINITY;
     for (int kb = 1; kb <= nB; ++kb) {
         const int tb = (nB + kb - 1) / kb;
@@ -235,7 +237,7 @@ lsp::Tile pair_tile(const lsp_grid* g)
             for (const int ch : {2, 4, 6, 8, 10, 12, 16, 20, 26, 34, 50, 66, 102}) {
                 if (ch > nS + 1) break;
                 const long long ctas = plane_ctas * ((nS + ch - 1) / ch);
-                const long long per_sm = (ctas + lsp::sm_count() - 1) / lsp::sm_count();
+                const long long per_sm = (ctas + sms - 1) / sms;
                 const long long waves = (per_sm + resident - 1) / resident;
                 const double cost = (0.5 * ch + 0.1) * (per_sm * weight + 5.0 * waves);
                 if (cost < best_cost || (cost == best_cost && tb * ta > best.tb * best.ta)) {

@@ -31,8 +31,8 @@
 //
 // Measured (GB300, us per stage of whole solves; default tile of the scalar
 // body before, its autotuned tile or run kernel in brackets, this kernel's
-// default tile now): rockets 300^3 ENO2 388 (182), 169; 100^3 20.8 (14.3),
-// 8.7; car4d 81^4 ENO3 870 (650), 438; 33 x 41 x 37 x 29 48, 21.5.  What
+// default tile now): rockets 300^3 ENO2 388 (182), 160; 100^3 20.8 (14.3),
+// 8.5; car4d 81^4 ENO3 870 (650), 438; 33 x 41 x 37 x 29 48, 21.5.  What
 // bounds it: instruction issue (51 % of the cycles, 150 instructions per node
 // in 3-D and 219 in 4-D, of which 45 and 125 are the scheme's arithmetic) and
 // the latency of the loads between barriers.
@@ -243,13 +243,13 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
         ha[k] = (a.alpha_from_ctl ? float(__longlong_as_double((long long)a.ctl->alpha_bits[k]))
                                   : a.alpha[k]) *
                 0.5f;
-    // axis k's share of a node's costate and dissipation from dx p-, dx p+,
+    // axis k's central costate and p+ - p- of a node from dx p-, dx p+,
     // rounded as the scalar body's (p+ + p-) / 2 and p+ - p- are compiled: the
     // product of p- fused into the sum and the difference
-    auto axis = [&](int k, float am, float ap, float& pbar, float& diss) {
+    auto axis = [&](int k, float am, float ap, float& pbar) -> float {
         const float pp = __fmul_rn(ap, a.inv_dx[k]);
         pbar = 0.5f * __fmaf_rn(am, a.inv_dx[k], pp);
-        diss = rfma(ha[k], __fmaf_rn(-am, a.inv_dx[k], pp), diss);
+        return __fmaf_rn(-am, a.inv_dx[k], pp);
     };
 
     // plane of the lead value j (beyond the end of an extrapolated axis the
@@ -351,10 +351,29 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
                 center[q][r] = m[q][r].u[0];
                 float pm, pp;
                 col_step<SCHEME>(m[q][r], lead[q][r], pm, pp);
-                diss[q][r] = 0.0f;
-                axis(AS, pm, pp, pbar[q][r][AS], diss[q][r]);
+                diss[q][r] = ha[AS] * axis(AS, pm, pp, pbar[q][r][AS]);
                 lead[q][r] = nlead[q][r];
             }
+        // Axis B is evaluated before A in 3-D, its dissipation added after A's
+        // (fewer live values: rockets 300^3 1921 against 2033 us for 6 steps),
+        // and after it in 4-D (car4d 81^4 2626 against 2684 us for 2 steps).
+        float bdiss[R0][RA];
+        auto axis_b = [&]() {
+#pragma unroll
+            for (int q = 0; q < R0; ++q)
+#pragma unroll
+                for (int r = 0; r < RA; ++r) {
+                    const float* p = cur + q * slab_floats + mine + r * P;
+                    float w[2 * G + 1], pm, pp;
+#pragma unroll
+                    for (int k = 0; k <= 2 * G; ++k) w[k] = k == G ? center[q][r] : p[k - G];
+                    eno_line<SCHEME, 1>(w, &pm, &pp);
+                    const float e = axis(AB, pm, pp, pbar[q][r][AB]);
+                    if constexpr (NDIM == 3) bdiss[q][r] = e;
+                    else diss[q][r] = rfma(ha[AB], e, diss[q][r]);
+                }
+        };
+        if constexpr (NDIM == 3) axis_b();
         // axis A
 #pragma unroll
         for (int q = 0; q < R0; ++q) {
@@ -365,20 +384,15 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
                 w[k] = k < G || k >= G + RA ? p[k * P] : center[q][(k - G) & (RA - 1)];
             eno_line<SCHEME, RA>(w, pm, pp);
 #pragma unroll
-            for (int r = 0; r < RA; ++r) axis(AA, pm[r], pp[r], pbar[q][r][AA], diss[q][r]);
+            for (int r = 0; r < RA; ++r)
+                diss[q][r] = rfma(ha[AA], axis(AA, pm[r], pp[r], pbar[q][r][AA]), diss[q][r]);
         }
-        // axis B
+        if constexpr (NDIM == 4) {
+            axis_b();
+        } else {
 #pragma unroll
-        for (int q = 0; q < R0; ++q)
-#pragma unroll
-            for (int r = 0; r < RA; ++r) {
-                const float* p = cur + q * slab_floats + mine + r * P;
-                float w[2 * G + 1], pm, pp;
-#pragma unroll
-                for (int k = 0; k <= 2 * G; ++k) w[k] = k == G ? center[q][r] : p[k - G];
-                eno_line<SCHEME, 1>(w, &pm, &pp);
-                axis(AB, pm, pp, pbar[q][r][AB], diss[q][r]);
-            }
+            for (int r = 0; r < RA; ++r) diss[0][r] = rfma(ha[AB], bdiss[0][r], diss[0][r]);
+        }
         // axis 0
         if constexpr (NDIM == 4) {
 #pragma unroll
@@ -392,7 +406,8 @@ __global__ void __launch_bounds__(kMarchThreads, MINB)
                 if (edge0) fix_extrapolated<R0, G>(w, o0, a.n[0]);
                 eno_line<SCHEME, R0>(w, pm, pp);
 #pragma unroll
-                for (int q = 0; q < R0; ++q) axis(0, pm[q], pp[q], pbar[q][r][0], diss[q][r]);
+                for (int q = 0; q < R0; ++q)
+                    diss[q][r] = rfma(ha[0], axis(0, pm[q], pp[q], pbar[q][r][0]), diss[q][r]);
             }
         }
         // Hamiltonian, rate, RK combination, tube
