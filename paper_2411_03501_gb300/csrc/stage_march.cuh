@@ -33,9 +33,9 @@
 // body before, its autotuned tile or run kernel in brackets, this kernel's
 // default tile now): rockets 300^3 ENO2 388 (182), 160; 100^3 20.8 (14.3),
 // 8.5; car4d 81^4 ENO3 870 (650), 438; 33 x 41 x 37 x 29 48, 21.5.  What
-// bounds it: instruction issue (51 % of the cycles, 150 instructions per node
-// in 3-D and 219 in 4-D, of which 45 and 125 are the scheme's arithmetic) and
-// the latency of the loads between barriers.
+// bounds it: instruction issue (65 % of the cycles on rockets 200^3, 165
+// instructions per node in 3-D and 244 in 4-D, of which 45 and 125 are the
+// scheme's arithmetic) and the latency of the loads between barriers.
 // Measured and not kept: 4 rows per thread (128 registers, fewer warps: 10.1
 // against 9.5 us at 100^3, 26.7 against 22.5 on the 4-D grid above); reading
 // every neighbour through L1 without staging (250 us at 300^3, 1580 at 81^4);
