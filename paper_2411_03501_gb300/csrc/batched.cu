@@ -83,14 +83,6 @@ cudaError_t launch_batched_persistent(int scheme, const BatchProblem* probs, con
                                    done, pc, ctl, wait_ns, s);
 }
 
-bool batch_tile_dims(int shape, int* tb, int* ta)
-{
-    if (shape < 0 || shape >= kBatchNumShapes) return false;
-    *tb = kBatchShapes[shape][0];
-    *ta = kBatchShapes[shape][1];
-    return true;
-}
-
 bool batch_supported(int ndim, int dyn)
 {
     if (ndim == 2) return dyn == NORMAL_SPEED || dyn == TRANSLATE || dyn == DOUBLE_INT;

@@ -1,6 +1,7 @@
 // batched.h -- the per-problem descriptor of a batched solve, shared by the
 // host layer (which builds the table) and the batched stage kernel.
 #pragma once
+#include "batch_plan.h"
 #include "lsp_internal.h"
 
 namespace lsp {
@@ -19,12 +20,9 @@ struct BatchProblem {
     int tb, ta;                 // tile of the two fastest axes (tb x ta = kBatchThreads)
 };
 
-// Every batched CTA has kBatchThreads threads; each problem's tile of its two
-// fastest axes is one of kBatchShapes (chosen per problem dimension by
-// lsp_solve_opts.batch_tiles), thread t covering (t % tb, t / tb).
+// Every batched CTA has kBatchThreads threads, thread t covering (t % tb,
+// t / tb) of its problem's tile (kBatchShapes, batch_plan.h).
 constexpr int kBatchThreads = 256;
-constexpr int kBatchNumShapes = 3;
-constexpr int kBatchShapes[kBatchNumShapes][2] = {{16, 16}, {32, 8}, {64, 4}};
 // the largest haloed tile of the shapes, in floats, for ghost width G
 __host__ __device__ constexpr int batch_max_tile(int G)
 {

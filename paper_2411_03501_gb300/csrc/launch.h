@@ -92,9 +92,6 @@ cudaError_t launch_batched_persistent(int scheme, const BatchProblem* probs, con
                                       unsigned int* done, PersistCtl* pc, Ctl* ctl,
                                       unsigned long long wait_ns, bool local, int cls,
                                       cudaStream_t s);
-// Tile shape `shape` (0: 16 x 16, 1: 32 x 8, 2: 64 x 4) of batched problems;
-// false for other values.
-bool batch_tile_dims(int shape, int* tb, int* ta);
 bool batch_supported(int ndim, int dyn);
 
 // Implicit-surface primitives and set operations (shapes.cu).

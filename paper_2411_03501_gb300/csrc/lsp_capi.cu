@@ -11,6 +11,7 @@
 
 #include "../../include/lsp.h"
 #include "adjoint.cuh"
+#include "batch_plan.h"
 #include "batched.h"
 #include "launch.h"
 #include "stage_generic.cuh"
@@ -1195,91 +1196,42 @@ size_t batch_persist_bytes(int nprob)
 // Test hook of the persistent batched launch (lsp_debug_stall_problem).
 int g_stall_problem = -1;
 
-// Planes per CTA when opts->batch_chunk is 0.  A stage of the whole batch has
-// x = (tiles x planes) / (3 CTAs x SMs) planes for each resident CTA: with
-// whole columns per CTA a small batch leaves most of them idle and waits for
-// the largest problem's column, with short chunks the persistent launch pays
-// its per-item overhead (counter, fences, dependency poll) and every CTA its
-// start more often.  Best of 4 .. 128 planes in milliseconds, against the
-// whole columns (128) used before, half 2-D fronts and half 3-D games, WENO5
-// RK3 (persistent; graph form in brackets):
-//   24 problems, x = 97: 32 planes 3.91, 128 5.06 (24: 4.04, 5.81)
-//   8 problems, x = 33: 16 planes 1.20, 2.69 (8: 1.25, 3.28)
-//   32 at half size, x = 21: 12 planes 0.92, 1.93 (8: 1.04, 2.30)
-//   4 at 0.4 size, x = 1: 4 planes 0.31, 1.06 (4: 0.34, 1.09)
-//   96 problems, x = 390: 128 planes 8.97 (32: 9.25, 64: 9.29, 128: 9.89)
-// which 5 + 0.31 x (persistent) and 4 + 0.2 x (graph) meet within 3 %.
-int batch_auto_chunk(int nprob, lsp_grid* const* grids, const lsp_solve_opts* o, int persistent)
-{
-    const bool local = o->diss != LSP_DISS_GLF || o->varform;
-    double planes = 0.0;
-    for (int i = 0; i < nprob; ++i) {
-        const lsp_grid* g = grids[i];
-        const int d = g->ndim;
-        int tb = 16, ta = 16;
-        lsp::batch_tile_dims(local ? 0 : (o->batch_tiles >> (2 * (d - 2))) & 3, &tb, &ta);
-        planes += (double)((g->n[d - 1] + tb - 1) / tb) * ((g->n[d - 2] + ta - 1) / ta) *
-                  (d >= 3 ? g->n[d - 3] : 1) * (d == 4 ? g->n[0] : 1);
-    }
-    const double x = planes / (3.0 * lsp::sm_count());
-    const double c = persistent ? 5.0 + 0.31 * x : 4.0 + 0.2 * x;
-    return c >= 128.0 ? 128 : std::max(4, (int)c / 2 * 2);
-}
-
 // Tile grid and field sizes of every problem; the total workspace bytes.
-// any_shape: size the block table for the largest tile count over every
-// shape (a workspace that serves any opts->batch_tiles).
+// any_shape: size the block table for every choice of tiles and chunk (a
+// workspace that serves any opts->batch_tiles and either form of the solve).
 void batch_geometry(int nprob, lsp_grid* const* grids, const lsp_solve_opts* o,
                     std::vector<BatchPlanEntry>& plan, size_t* bytes, long long* total_blocks,
                     bool any_shape = false)
 {
-    const int chunk = o->batch_chunk > 0 ? o->batch_chunk
-                                         : batch_auto_chunk(nprob, grids, o, o->batch_persistent);
-    // a workspace sized for either form of the solve
-    const int finest = o->batch_chunk > 0 ? chunk
-                                          : std::min(batch_auto_chunk(nprob, grids, o, 0),
-                                                     batch_auto_chunk(nprob, grids, o, 1));
+    const bool local = o->diss != LSP_DISS_GLF || o->varform;
+    double planes = 0.0;
+    for (int i = 0; i < nprob; ++i)
+        planes += lsp::batch_planes(grids[i]->ndim, grids[i]->n,
+                                    lsp::batch_shape(o->batch_tiles, grids[i]->ndim, local));
+    const int chunk = o->batch_chunk > 0
+                          ? o->batch_chunk
+                          : lsp::batch_auto_chunk(planes, lsp::sm_count(), o->batch_persistent != 0);
     plan.resize(nprob);
     size_t fields = 0;
     long long blocks = 0;
     for (int i = 0; i < nprob; ++i) {
         const lsp_grid* g = grids[i];
         BatchPlanEntry& e = plan[i];
-        const int d = g->ndim;
         e.p = i;
         e.nsteps = 0;
         e.dt = e.dt_last = 0.0;
-        // the local-coefficient / clipped kernels are compiled for 16 x 16 tiles
-        const bool local = o->diss != LSP_DISS_GLF || o->varform;
-        const int shape = local ? 0 : (o->batch_tiles >> (2 * (d - 2))) & 3;
-        long long nb_max = 0;
-        for (int sh = 0; sh < 3; ++sh) {
-            if (!any_shape && sh != shape) continue;
-            int tb = 16, ta = 16;
-            lsp::batch_tile_dims(sh, &tb, &ta);
-            const int nbx = (g->n[d - 1] + tb - 1) / tb, nby = (g->n[d - 2] + ta - 1) / ta;
-            int ch = 1, nchunks = 1;
-            if (d >= 3) {
-                const int nS = g->n[d - 3];
-                ch = std::min(chunk, nS);
-                nchunks = (nS + ch - 1) / ch;
-            }
-            const long long nb = (long long)nbx * nby * nchunks * (d == 4 ? g->n[0] : 1);
-            const int fine = d >= 3 ? (g->n[d - 3] + finest - 1) / finest : 1;
-            nb_max = std::max(nb_max, nb / nchunks * std::max(fine, nchunks));
-            if (sh == shape) {
-                e.tb = tb;
-                e.ta = ta;
-                e.nbx = nbx;
-                e.nby = nby;
-                e.ch = ch;
-                e.nchunks = nchunks;
-                e.nblocks = (int)nb;
-            }
-        }
+        const lsp::BatchTiling t =
+            lsp::batch_tiling(g->ndim, g->n, lsp::batch_shape(o->batch_tiles, g->ndim, local), chunk);
+        e.tb = t.tb;
+        e.ta = t.ta;
+        e.nbx = t.nbx;
+        e.nby = t.nby;
+        e.ch = t.ch;
+        e.nchunks = t.nchunks;
+        e.nblocks = (int)t.blocks;
         e.field_bytes = round256((size_t)g->npts * sizeof(float));
         fields += nfields(o->rk_order) * e.field_bytes;
-        blocks += any_shape ? nb_max : e.nblocks;
+        blocks += any_shape ? lsp::batch_max_blocks(g->ndim, g->n, o->batch_chunk) : e.nblocks;
     }
     *total_blocks = blocks;
     *bytes = lsp::kCtlBytes + round256((size_t)nprob * sizeof(lsp::BatchProblem)) +

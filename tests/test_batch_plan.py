@@ -1,0 +1,86 @@
+"""The cut of a batched solve into CTAs (csrc/batch_plan.h, host arithmetic):
+a workspace sized once holds the CTA table of every tile choice, both launch
+forms and local coefficients, and of the same batch without some problems."""
+import ctypes
+import os
+import random
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_2411_03501_gb300", "csrc")
+SHIM = r"""
+#include "batch_plan.h"
+using namespace lsp;
+extern "C" long long sized(int np, const int* nd, const int (*n)[4], int chunk)
+{
+    long long b = 0;
+    for (int i = 0; i < np; ++i) b += batch_max_blocks(nd[i], n[i], chunk);
+    return b;
+}
+extern "C" long long needed(int np, const int* nd, const int (*n)[4], int tiles, int chunk,
+                            int persistent, int local, int sms)
+{
+    double planes = 0;
+    for (int i = 0; i < np; ++i) planes += batch_planes(nd[i], n[i], batch_shape(tiles, nd[i], local));
+    if (chunk <= 0) chunk = batch_auto_chunk(planes, sms, persistent);
+    long long b = 0;
+    for (int i = 0; i < np; ++i) b += batch_tiling(nd[i], n[i], batch_shape(tiles, nd[i], local), chunk).blocks;
+    return b;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plan")
+    (d / "shim.cpp").write_text(SHIM)
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(d / "shim.cpp"), "-o",
+                    str(d / "shim.so")], check=True)
+    lib = ctypes.CDLL(str(d / "shim.so"))
+    lib.sized.restype = lib.needed.restype = ctypes.c_longlong
+
+    def args(grids):
+        n = len(grids)
+        return n, (ctypes.c_int * n)(*map(len, grids)), \
+            ((ctypes.c_int * 4) * n)(*[(ctypes.c_int * 4)(*g) for g in grids])
+    return (lambda g, chunk: lib.sized(*args(g), chunk),
+            lambda g, tiles, chunk, pers, local, sms: lib.needed(*args(g), tiles, chunk, pers, local, sms))
+
+
+def _batches():
+    yield [[98, 115, 94]]
+    yield [[115, 98, 96]]
+    yield [[192, 89, 35]]
+    rng = random.Random(5)
+    top = {2: 700, 3: 200, 4: 50}
+    for _ in range(300):
+        yield [[int(7 * (top[d] / 7) ** rng.random()) for _ in range(d)]
+               for d in rng.choices([2, 3, 4], k=rng.choice([1, 1, 2, 5, 12]))]
+
+
+@pytest.mark.parametrize("sms", [1, 148, 152])
+def test_one_workspace_serves_every_tile_choice(plan, sms):
+    sized, needed = plan
+    rng = random.Random(6)
+    for grids in _batches():
+        some = rng.sample(grids, rng.randint(1, len(grids)))
+        for chunk in (0, 17):
+            room = sized(grids, chunk)
+            for t2 in range(3):
+                for t3 in range(3):
+                    for t4 in range(3):
+                        for pers in (0, 1):
+                            for g in (grids, some):
+                                tiles = t2 | t3 << 2 | t4 << 4
+                                assert needed(g, tiles, chunk, pers, 0, sms) <= room, (g, tiles, chunk)
+                                assert needed(g, tiles, chunk, pers, 1, sms) <= room, (g, tiles, chunk)
+
+
+def test_chunks_by_work_stay_in_their_range(plan):
+    """One CTA's column of a tiny batch is cut into 4 planes, a huge batch's
+    into 128."""
+    _, needed = plan
+    assert needed([[64, 16, 16]], 0, 0, 0, 0, 152) == 16
+    assert needed([[128, 16, 16]] * 4000, 0, 0, 1, 0, 152) == 4000

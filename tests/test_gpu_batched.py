@@ -217,3 +217,27 @@ def test_batched_autotune_picks_valid_tiles_and_leaves_fields():
     with pytest.raises(B.LspError) as e:
         B.Batch(specs, tiles=0b11)
     assert e.value.status == B.LSP_EINVAL
+
+
+@pytest.mark.parametrize("n", [[98, 115, 94], [115, 98, 96], [192, 89, 35]])
+def test_one_workspace_serves_every_tile_shape_and_form(n):
+    """The workspace sized at one batch_tiles value serves the others, with
+    the planes per CTA chosen by the batch's work, and gives the field of a
+    workspace sized at theirs."""
+    spec = dict(W.air3d(nx=n)[0], tube=False)
+    phi = to_dev(rounded(W.smooth_field(spec, seed=8), "f32"), "f32")
+    ref = {}
+    for sized in range(3):
+        Bt = B.Batch([spec], use_graph=False, tiles=sized << 2)
+        t = [1.5 * B.lsp_cfl_dt(Bt.grids[0], Bt.opts, 0.0, 1e9)]
+        for shape in range(3):
+            for persistent in (False, True):
+                if sized == 0:
+                    x = phi.clone()
+                    B.Batch([spec], use_graph=False, tiles=shape << 2, persistent=persistent).solve([x], t_final=t)
+                    ref[shape, persistent] = x
+                Bt.opts.batch_tiles, Bt.opts.batch_persistent = shape << 2, int(persistent)
+                x = phi.clone()
+                assert Bt.solve([x], t_final=t)[0]["steps"] == 2
+                assert torch.equal(x, ref[shape, persistent])
+    assert Bt.autotune([phi], t_final=t) in (0, 4, 8)
