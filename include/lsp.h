@@ -286,7 +286,8 @@ lsp_status lsp_hj_solve(lsp_grid* grid, const lsp_solve_opts* opts, void* phi,
  *        with a 2-cell halo 3 (checked for ENO2; a step whose scheme's
  *        halo does not fit runs the generic kernel), or pair is 6 with at
  *        most 256 threads, the tile's frame (2 halo (tb + ta) values) in 2
- *        values per thread and fewer than 2^30 nodes.
+ *        values per thread (checked for ENO2, as for pair 5) and fewer than
+ *        2^30 nodes.
  * lsp_get_tile reports the tile a step with `opts` would use (all -1 when
  * the generic kernel runs). */
 lsp_status lsp_set_tile(lsp_grid* grid, int tb, int ta, int ch, int minb, int pair);

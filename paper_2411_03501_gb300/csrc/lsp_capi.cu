@@ -911,7 +911,7 @@ lsp_status lsp_set_tile(lsp_grid* g, int tb, int ta, int ch, int minb, int pair)
     lsp::Tile t{tb, ta, ch, minb, pair};
     // validated for a scheme that has the variant (the step re-checks the
     // tile against its own scheme and runs the generic kernel if it fails)
-    if (!lsp::tile_valid(g->ndim, pair == 5 ? LSP_ENO2 : (pair >= 3 ? LSP_ENO3 : LSP_WENO5), t,
+    if (!lsp::tile_valid(g->ndim, pair >= 5 ? LSP_ENO2 : (pair >= 3 ? LSP_ENO3 : LSP_WENO5), t,
                          g->n))
         return fail(LSP_EINVAL, "tile %dx%dx%d (%d CTAs/SM) is not valid for this grid", tb, ta,
                     ch, minb);
