@@ -79,6 +79,19 @@ bool run_tile_ok(int ndim, int scheme, int run, int tb, int ta)
     return ta >= 1 && tbt * ta <= 256 && 2 * sizeof(float) * floats <= kRunMaxSmem;
 }
 
+// One node per thread in the chunks of a run or march tile.  A march's blocks
+// hold 2 slabs of axis 0 (4-D), these one: longer chunks where the launch
+// would pass 65535 z-blocks; ch = 0 when no chunk avoids that.
+static Tile local_tile(int ndim, const Tile& t, const int* n)
+{
+    Tile l{32, 8, t.ch, 3, 0};
+    const int nS = n[ndim - 3], outer = ndim == 4 ? n[0] : 1;
+    const int most = 65535 / outer;  // chunks
+    if (most < 1 || (n[ndim - 2] + l.ta - 1) / l.ta > 65535) l.ch = 0;
+    else if ((nS + l.ch - 1) / l.ch > most) l.ch = (nS + most - 1) / most;
+    return l;
+}
+
 cudaError_t launch_stage_tiled(int ndim, int scheme, int dyn, const StageArgs<float>& a,
                                const Tile& t, cudaStream_t s)
 {
@@ -88,9 +101,11 @@ cudaError_t launch_stage_tiled(int ndim, int scheme, int dyn, const StageArgs<fl
     if ((a.local_alpha || a.varform) && !(scheme == WENO5 && t.pair == 2 && dyn != QUADRATIC)) {
         // the face-shared runs and marches have no local variant: a one-node-per-thread
         // tile of the same chunking runs the local body
-        const Tile tl = (t.pair == 3 || t.pair == 4 || t.pair == 6) ? Tile{32, 8, t.ch, 3, 0}
-                                                     : Tile{t.tb, t.ta, t.ch, t.minb, 0};
-        return launch_stage_tiled_local(ndim, scheme, dyn, a, tl, s);
+        if (t.pair != 3 && t.pair != 4 && t.pair != 6)
+            return launch_stage_tiled_local(ndim, scheme, dyn, a, Tile{t.tb, t.ta, t.ch, t.minb, 0}, s);
+        const Tile tl = local_tile(ndim, t, a.n);
+        return tl.ch > 0 ? launch_stage_tiled_local(ndim, scheme, dyn, a, tl, s)
+                         : launch_stage<float>(ndim, scheme, dyn, a, s);
     }
     if (t.pair == 5) {  // a single stage on a fused-RK2 tile: the scalar body
         const Tile ts{t.tb, t.ta, t.ch, t.minb, 0};
