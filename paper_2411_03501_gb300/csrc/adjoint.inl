@@ -22,11 +22,9 @@ template <int NDIM, int SCHEME, int DYN>
 static cudaError_t launch_pass_a(const AdjArgs<LSP_REAL>& a, cudaStream_t s)
 {
     constexpr size_t smem = adj_a_smem_bytes<NDIM, LSP_REAL>();
+    if (const cudaError_t e = allow_smem(adj_stage_a<NDIM, SCHEME, DYN, LSP_REAL>, smem, smem)) return e;
     static const int resident = [] {
         int nsm = sm_count(), per = 1;
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute(adj_stage_a<NDIM, SCHEME, DYN, LSP_REAL>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                 &per, adj_stage_a<NDIM, SCHEME, DYN, LSP_REAL>, 256, smem) != cudaSuccess || per < 1)
             per = 1;

@@ -25,6 +25,18 @@ cudaError_t launch_dependent(void (*fn)(P...), dim3 grid, dim3 block, size_t sme
     return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
 }
 
+// Lets a kernel take more dynamic shared memory than every launch may (48 KB);
+// called before each launch, since the attribute belongs to the current
+// device.  The limit set is the same for every launch of a kernel, so threads
+// that launch it do not lower one another's.
+template <typename F>
+cudaError_t allow_smem(F* fn, size_t smem, size_t most)
+{
+    if (smem <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(reinterpret_cast<const void*>(fn),
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 struct GridGeom;
 
 // Fused stage (generic one-thread-per-node kernel).

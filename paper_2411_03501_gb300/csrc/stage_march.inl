@@ -21,9 +21,6 @@ cudaError_t march_launch(const StageArgs<float>& a, const Tile& t, cudaStream_t 
               nchunks * (ND == 4 ? (a.n[0] + R0 - 1) / R0 : 1));
     const size_t smem = 2 * sizeof(float) * R0 * (t.ta + 2 * G) * kMarchPitch;
     const int threads = march_threads(t);
-    const auto prepare = [](auto* fn) {
-        return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunMaxSmem);
-    };
     // In 4-D a launch of many waves is faster as an ordinary one (car4d 81^4,
     // 27 planes, 6 waves: 434 us per stage against 503; 33 x 41 x 37 x 29, one
     // wave: 22.9 against 21.2).  In 3-D the dependent form is faster there too
@@ -33,15 +30,13 @@ cudaError_t march_launch(const StageArgs<float>& a, const Tile& t, cudaStream_t 
         const long long ctas = (long long)grid.x * grid.y * grid.z;
         if (ctas * threads > 4LL * kResident * sm_count()) {
             auto* fn = stage_march_kernel<ND, SCHEME, DYN, LSP_MARCH_MINB, false>;
-            static const cudaError_t attr = prepare(fn);
-            if (attr != cudaSuccess) return attr;
+            if (const cudaError_t e = allow_smem(fn, smem, kRunMaxSmem)) return e;
             fn<<<grid, threads, smem, s>>>(a, t.tb, t.ta, t.ch, nchunks);
             return cudaGetLastError();
         }
     }
     auto* fn = stage_march_kernel<ND, SCHEME, DYN, LSP_MARCH_MINB, true>;
-    static const cudaError_t attr = prepare(fn);
-    if (attr != cudaSuccess) return attr;
+    if (const cudaError_t e = allow_smem(fn, smem, kRunMaxSmem)) return e;
     return launch_dependent(fn, grid, threads, smem, s, a, t.tb, t.ta, t.ch, nchunks);
 }
 

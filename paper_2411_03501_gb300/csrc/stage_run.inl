@@ -22,9 +22,7 @@ cudaError_t run_launch(const StageArgs<float>& a, const Tile& t, cudaStream_t s)
     const size_t smem = 2 * sizeof(float) * (size_t)run_plane_floats<NDIM, SCHEME, R, TBT>(t.ta);
     if (smem > kRunMaxSmem) return cudaErrorInvalidValue;
     auto* fn = stage_run_kernel<NDIM, SCHEME, DYN, R, TBT, LSP_RUN_MINB>;
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunMaxSmem);
-    if (attr != cudaSuccess) return attr;
+    if (const cudaError_t e = allow_smem(fn, smem, kRunMaxSmem)) return e;
     fn<<<grid, block, smem, s>>>(a, t.ch, nchunks);
     return cudaGetLastError();
 }
