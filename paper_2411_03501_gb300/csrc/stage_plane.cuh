@@ -77,10 +77,26 @@ __device__ __forceinline__ double near_reciprocal(double e)
                                 (__double_as_longlong(e) & 0x7ff0000000000000ll));
 }
 
+// Power of two that scales q_k = s_k + eps of the WENO5 weights (plane_weno).
+// FP32: close to 1/max q_k, so that no product of weights passes 16; scaled by
+// 1/eps (eps <= q_k <= 4e7 eps) their products with the stencil values
+// overflow on rough data from undivided differences of 1e8 on.  FP64 has the
+// range for 1/eps, which is known earlier (max q_k costs 3.7 % of a stage there
+// and 1 % in FP32).
+__device__ __forceinline__ float weight_scale(float, float q1, float q2, float q3)
+{
+    return near_reciprocal(fmaxf(fmaxf(q1, q2), q3));
+}
+__device__ __forceinline__ double weight_scale(double eps, double, double, double)
+{
+    return near_reciprocal(eps);
+}
+
 // weno5_combine (stencil.cuh) with one division instead of four: the weights
-// alpha_k = c_k / q_k^2 are multiplied by (q_1 q_2 q_3)^2, after q_k = s_k + eps
-// has been scaled by a power of two close to 1/eps.  The scaling is exact and
-// keeps every product in range (eps <= q_k <= 4e7 eps).
+// alpha_k = c_k / q_k^2 are multiplied by (q_1 q_2 q_3)^2, after q_k has been
+// scaled by a power of two (exact).  Finite wherever the form with four
+// divisions is (in FP32 its squares overflow from differences of 1e9 on), up
+// to differences of 1e18 in FP32 and 1e150 in FP64.
 template <typename R>
 __device__ __forceinline__ R plane_weno(R v1, R v2, R v3, R v4, R v5, R floor_)
 {
@@ -95,8 +111,9 @@ __device__ __forceinline__ R plane_weno(R v1, R v2, R v3, R v4, R v5, R floor_)
     const R s3 = R(13.0 / 12.0) * a3 * a3 + R(0.25) * b3 * b3;
     const R m = mag_max(mag_max(mag_max(v1, v2), mag_max(v3, v4)), v5);
     const R eps = R(1e-6) * (m * m) + floor_;
-    const R sc = near_reciprocal(eps);
-    const R q1 = (s1 + eps) * sc, q2 = (s2 + eps) * sc, q3 = (s3 + eps) * sc;
+    const R t1 = s1 + eps, t2 = s2 + eps, t3 = s3 + eps;
+    const R sc = weight_scale(eps, t1, t2, t3);
+    const R q1 = t1 * sc, q2 = t2 * sc, q3 = t3 * sc;
     const R Q1 = q1 * q1, Q2 = q2 * q2, Q3 = q3 * q3;
     const R al1 = R(0.1) * (Q2 * Q3), al2 = R(0.6) * (Q1 * Q3), al3 = R(0.3) * (Q1 * Q2);
     return (al1 * phi1 + al2 * phi2 + al3 * phi3) / (al1 + al2 + al3);
