@@ -17,7 +17,7 @@ static inline int stage_blocks(long long npts)
 template <int SCHEME>
 static cudaError_t plane_dyn(int dyn, const StageArgs<LSP_REAL>& a, cudaStream_t s)
 {
-    const int nt = plane_block(a.npts), nb = (a.npts + nt - 1) / nt;
+    const int nt = plane_block(a.npts, sm_count()), nb = (a.npts + nt - 1) / nt;
     switch (dyn) {
     case NORMAL_SPEED: return launch_dependent(stage_plane_kernel<SCHEME, NORMAL_SPEED, LSP_REAL>, nb, nt, 0, s, a);
     case TRANSLATE: return launch_dependent(stage_plane_kernel<SCHEME, TRANSLATE, LSP_REAL>, nb, nt, 0, s, a);
@@ -88,7 +88,7 @@ cudaError_t launch_stage<LSP_REAL>(int ndim, int scheme, int dyn, const StageArg
 static cudaError_t prange_plane(int scheme, const StageArgs<LSP_REAL>& a, const StepChoice& ch,
                                 cudaStream_t s)
 {
-    const int nt = plane_block(a.npts), nb = (a.npts + nt - 1) / nt;
+    const int nt = plane_block(a.npts, sm_count()), nb = (a.npts + nt - 1) / nt;
     switch (scheme) {
     case UPWIND1: return launch_dependent(prange_plane_kernel<UPWIND1, LSP_REAL>, nb, nt, 0, s, a, ch);
     case ENO2: return launch_dependent(prange_plane_kernel<ENO2, LSP_REAL>, nb, nt, 0, s, a, ch);

@@ -37,6 +37,26 @@ cudaError_t allow_smem(F* fn, size_t smem, size_t most)
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
+// Threads per block of the 2-D kernels (stage_plane.cuh): the fewest nodes on
+// the busiest SM (whole warps, 64 to 256 threads; the larger block unless a
+// smaller one spares 1 %).  On large grids every size splits evenly, and
+// small blocks are bound by the rate at which blocks start (about one per ns:
+// 8192^2 FP32 first order in blocks of 64 threads 1056 us per stage, of 256
+// threads 357).
+inline int plane_block(long long npts, long long sms)
+{
+    int best = 256;
+    long long cost = -1;
+    for (int t = 256; t >= 64; t -= 32) {
+        const long long c = ((npts + t - 1) / t + sms - 1) / sms * t;
+        if (cost < 0 || c * 100 < cost * 99) {
+            cost = c;
+            best = t;
+        }
+    }
+    return best;
+}
+
 struct GridGeom;
 
 // Fused stage (generic one-thread-per-node kernel).

@@ -25,23 +25,6 @@
 
 namespace lsp {
 
-// Threads per block: the fewest nodes on the busiest SM (whole warps, 64 to
-// 256 threads; ties to the larger block).
-inline int plane_block(long long npts)
-{
-    const long long sms = sm_count();
-    int best = 64;
-    long long cost = -1;
-    for (int t = 64; t <= 256; t += 32) {
-        const long long c = ((npts + t - 1) / t + sms - 1) / sms * t;
-        if (cost < 0 || c <= cost) {
-            cost = c;
-            best = t;
-        }
-    }
-    return best;
-}
-
 // |a| <= |b| (false when either is NaN).
 __device__ __forceinline__ bool mag_le(float a, float b) { return fabsf(a) <= fabsf(b); }
 __device__ __forceinline__ unsigned long long mag_bits(double a)
