@@ -1,5 +1,7 @@
 // dispatch.inl -- explicit instantiation of the generic stage kernels for one
 // precision LSP_REAL (included by stage_f32.cu / stage_f64.cu).
+#include <algorithm>
+
 #include "launch.h"
 #include "stage_generic.cuh"
 #include "stage_plane.cuh"
@@ -17,12 +19,15 @@ static inline int stage_blocks(long long npts)
 template <int SCHEME>
 static cudaError_t plane_dyn(int dyn, const StageArgs<LSP_REAL>& a, cudaStream_t s)
 {
-    const int nt = plane_block(a.npts, sm_count()), nb = (a.npts + nt - 1) / nt;
+    const int nt = plane_block(a.npts, sm_count());
+    int nb = (a.npts + nt - 1) / nt;
+    if (sizeof(LSP_REAL) == 8) nb = std::min(nb, 16 * sm_count());
+    const PlaneConst<LSP_REAL> pc = plane_const(a);
     switch (dyn) {
-    case NORMAL_SPEED: return launch_dependent(stage_plane_kernel<SCHEME, NORMAL_SPEED, LSP_REAL>, nb, nt, 0, s, a);
-    case TRANSLATE: return launch_dependent(stage_plane_kernel<SCHEME, TRANSLATE, LSP_REAL>, nb, nt, 0, s, a);
-    case QUADRATIC: return launch_dependent(stage_plane_kernel<SCHEME, QUADRATIC, LSP_REAL>, nb, nt, 0, s, a);
-    case DOUBLE_INT: return launch_dependent(stage_plane_kernel<SCHEME, DOUBLE_INT, LSP_REAL>, nb, nt, 0, s, a);
+    case NORMAL_SPEED: return launch_dependent(stage_plane_kernel<SCHEME, NORMAL_SPEED, LSP_REAL>, nb, nt, 0, s, a, pc);
+    case TRANSLATE: return launch_dependent(stage_plane_kernel<SCHEME, TRANSLATE, LSP_REAL>, nb, nt, 0, s, a, pc);
+    case QUADRATIC: return launch_dependent(stage_plane_kernel<SCHEME, QUADRATIC, LSP_REAL>, nb, nt, 0, s, a, pc);
+    case DOUBLE_INT: return launch_dependent(stage_plane_kernel<SCHEME, DOUBLE_INT, LSP_REAL>, nb, nt, 0, s, a, pc);
     }
     return cudaErrorInvalidValue;
 }
@@ -89,11 +94,12 @@ static cudaError_t prange_plane(int scheme, const StageArgs<LSP_REAL>& a, const 
                                 cudaStream_t s)
 {
     const int nt = plane_block(a.npts, sm_count()), nb = (a.npts + nt - 1) / nt;
+    const PlaneConst<LSP_REAL> pc = plane_const(a);
     switch (scheme) {
-    case UPWIND1: return launch_dependent(prange_plane_kernel<UPWIND1, LSP_REAL>, nb, nt, 0, s, a, ch);
-    case ENO2: return launch_dependent(prange_plane_kernel<ENO2, LSP_REAL>, nb, nt, 0, s, a, ch);
-    case ENO3: return launch_dependent(prange_plane_kernel<ENO3, LSP_REAL>, nb, nt, 0, s, a, ch);
-    case WENO5: return launch_dependent(prange_plane_kernel<WENO5, LSP_REAL>, nb, nt, 0, s, a, ch);
+    case UPWIND1: return launch_dependent(prange_plane_kernel<UPWIND1, LSP_REAL>, nb, nt, 0, s, a, pc, ch);
+    case ENO2: return launch_dependent(prange_plane_kernel<ENO2, LSP_REAL>, nb, nt, 0, s, a, pc, ch);
+    case ENO3: return launch_dependent(prange_plane_kernel<ENO3, LSP_REAL>, nb, nt, 0, s, a, pc, ch);
+    case WENO5: return launch_dependent(prange_plane_kernel<WENO5, LSP_REAL>, nb, nt, 0, s, a, pc, ch);
     }
     return cudaErrorInvalidValue;
 }

@@ -10,13 +10,18 @@
 //  - index arithmetic is 32-bit, and all loads are requested at once:
 //    windows next to an edge load wrapped or clamped nodes and have their
 //    ghosts (Sec. III-B) replaced in registers;
-//  - FP64 magnitude comparisons, maxima and the finiteness test run on the
-//    bits of the values in the integer pipe, and WENO5 divides once per side
-//    instead of four times.  Otherwise the operations and their order are the
-//    generic kernel's (ENO2 and ENO3 give its bits).
+//  - FP64 maxima and the finiteness test run on the bits of the values in the
+//    integer pipe, the launch's constants come from the host (PlaneConst),
+//    and WENO5 divides once per side instead of four times.  Otherwise the
+//    operations and their order are the generic kernel's (ENO2 and ENO3 give
+//    its bits).
 // Measured (GB300, us per stage of whole solves, generic kernel before):
-// 101 x 101 FP64 ENO2 6.4, 4.8; 127 x 93 FP64 WENO5 31.8, 14.6; 513 x 401
-// FP64 WENO5 174, 135 (the FP64 pipe); 301 x 177 FP32 WENO5 4.4, 3.5.  The
+// 101 x 101 FP64 ENO2 8.7, 5.0; 127 x 93 FP64 WENO5 31.8, 13.6; 513 x 401
+// FP64 WENO5 176, 128 (the FP64 pipe); 301 x 177 FP32 WENO5 6.6, 3.9; 4096^2
+// FP32 first order 179, 93, WENO5 436, 276; 4096^2 FP64 first order 1019,
+// 1014, ENO2 1596, 1642, ENO3 2474, 2485, WENO5 11470, 9720 (84 % of the FP64
+// pipe; ENO2 executes one FP64 instruction more per axis than the generic
+// kernel, found in the counters and not explained).  The
 // Jiang-Peng form of WENO5 (stage_tiled.cuh) with one division takes 10-15 %
 // less in FP64, but its error against FP64 torch was 2-15 % above the
 // generic kernel's on four cases and it was not kept.
@@ -26,15 +31,11 @@
 namespace lsp {
 
 // |a| <= |b| (false when either is NaN).
-__device__ __forceinline__ bool mag_le(float a, float b) { return fabsf(a) <= fabsf(b); }
+template <typename R>
+__device__ __forceinline__ bool mag_le(R a, R b) { return rabs(a) <= rabs(b); }
 __device__ __forceinline__ unsigned long long mag_bits(double a)
 {
     return (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
-}
-__device__ __forceinline__ bool mag_le(double a, double b)
-{
-    const unsigned long long ia = mag_bits(a), ib = mag_bits(b);
-    return ia <= ib && ib <= 0x7ff0000000000000ull;
 }
 // max(|a|, |b|) of finite values (a NaN operand gives NaN)
 __device__ __forceinline__ float mag_max(float a, float b) { return fmaxf(fabsf(a), fabsf(b)); }
@@ -149,47 +150,80 @@ __device__ __forceinline__ void plane_window(const R* p, int c, int n, int s,
     if (!inside && !periodic) fix_extrapolated<1, G>(u, c, n);
 }
 
+// Constants of a launch, formed on the host: a thread has few nodes, and what
+// it forms once costs FP64 operations (101 x 101 FP64 ENO2 4.6 -> 4.4 us per
+// stage of a graph; 2048^2 FP64 first order 282 -> 264).
+template <typename R>
+struct PlaneConst {
+    R cl;         // c_l dt (dt not from the control block)
+    R half[2];    // alpha / 2 (alpha not from the control block)
+    R floor_[2];  // floor of WENO5's epsilon
+};
+
+template <typename R>
+PlaneConst<R> plane_const(const StageArgs<R>& a)
+{
+    PlaneConst<R> p;
+    p.cl = a.c_l * a.dt;
+    for (int k = 0; k < 2; ++k) {
+        p.half[k] = a.alpha[k] * R(0.5);
+        p.floor_[k] = Num<R>::eps_floor(a.inv_dx[k]);
+    }
+    return p;
+}
+
+// A thread takes one node (FP32) or the nodes of a grid-stride loop (FP64, at
+// most 16 blocks per SM: 4096^2 first order 1038 us in one pass of blocks,
+// 1014 in the loop).
 template <int SCHEME, int DYN, typename R>
-__global__ void __launch_bounds__(256) stage_plane_kernel(StageArgs<R> a)
+__global__ void __launch_bounds__(256) stage_plane_kernel(StageArgs<R> a, PlaneConst<R> pc)
 {
     constexpr int G = ghost_width(SCHEME);
-    const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = (int)(idx / (unsigned)a.n[1]), j = (int)(idx - (unsigned)i * (unsigned)a.n[1]);
+    unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
+    int i = (int)(idx / (unsigned)a.n[1]), j = (int)(idx - (unsigned)i * (unsigned)a.n[1]);
     stage_wait();
     stage_release();
     if (idx >= (unsigned)a.npts || past_last_step(a)) return;
-    R u[2][2 * G + 1];
-    plane_window<G>(a.phi_s + idx, i, a.n[0], a.stride[0], a.periodic[0], u[0]);
-    plane_window<G>(a.phi_s + idx, j, a.n[1], 1, a.periodic[1], u[1]);
-    const R vn = a.phi_n ? a.phi_n[idx] : R(0);
-    const R g = a.tube ? a.target[idx] : R(0);
-    const R dt = a.dt_from_ctl ? R(a.ctl->dt) : a.dt;
-    const R x[2] = {rfma(R(i), a.h[0], a.lo[0]), rfma(R(j), a.h[1], a.lo[1])};
-    R pbar[2], diss = R(0);
+    for (;;) {
+        R u[2][2 * G + 1];
+        plane_window<G>(a.phi_s + idx, i, a.n[0], a.stride[0], a.periodic[0], u[0]);
+        plane_window<G>(a.phi_s + idx, j, a.n[1], 1, a.periodic[1], u[1]);
+        const R vn = a.phi_n ? a.phi_n[idx] : R(0);
+        const R g = a.tube ? a.target[idx] : R(0);
+        const R cl = a.dt_from_ctl ? a.c_l * R(a.ctl->dt) : pc.cl;
+        const R x[2] = {rfma(R(i), a.h[0], a.lo[0]), rfma(R(j), a.h[1], a.lo[1])};
+        R pbar[2], diss = R(0);
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        R pm, pp;
-        plane_derivs<SCHEME>(u[k], Num<R>::eps_floor(a.inv_dx[k]), pm, pp);
-        pm *= a.inv_dx[k];
-        pp *= a.inv_dx[k];
-        R al = a.alpha_from_ctl ? R(__longlong_as_double((long long)a.ctl->alpha_bits[k])) : a.alpha[k];
-        if (a.local_alpha) al = local_alpha<DYN>(x, k, a.prm, R(0), R(1), pm, pp);
-        pbar[k] = R(0.5) * (pp + pm);
-        diss += al * R(0.5) * (pp - pm);
+        for (int k = 0; k < 2; ++k) {
+            R pm, pp;
+            plane_derivs<SCHEME>(u[k], pc.floor_[k], pm, pp);
+            pm *= a.inv_dx[k];
+            pp *= a.inv_dx[k];
+            R ha = pc.half[k];  // alpha / 2
+            if (a.alpha_from_ctl) ha = R(__longlong_as_double((long long)a.ctl->alpha_bits[k])) * R(0.5);
+            if (a.local_alpha) ha = local_alpha<DYN>(x, k, a.prm, R(0), R(1), pm, pp) * R(0.5);
+            pbar[k] = R(0.5) * (pp + pm);
+            diss += ha * (pp - pm);
+        }
+        const R H = hamiltonian<DYN, 2>(x, pbar, a.prm);
+        R L = -(H - diss);
+        if (a.varform) L = rmin(L, R(0));
+        R v = a.c_s * u[1][G] + cl * L;
+        if (a.phi_n) v += a.c_n * vn;
+        if (a.tube) v = rmin(v, g);
+        if (!is_finite_bits(v)) atomicOr(&a.ctl->flags, kFlagNonFinite);
+        a.out[idx] = v;
+        if constexpr (sizeof(R) == 4) return;
+        idx += gridDim.x * blockDim.x;  // below 2^31 + 2^23
+        if (idx >= (unsigned)a.npts) return;
+        i = (int)(idx / (unsigned)a.n[1]);
+        j = (int)(idx - (unsigned)i * (unsigned)a.n[1]);
     }
-    const R H = hamiltonian<DYN, 2>(x, pbar, a.prm);
-    R L = -(H - diss);
-    if (a.varform) L = rmin(L, R(0));
-    R v = a.c_s * u[1][G] + a.c_l * dt * L;
-    if (a.phi_n) v += a.c_n * vn;
-    if (a.tube) v = rmin(v, g);
-    if (!is_finite_bits(v)) atomicOr(&a.ctl->flags, kFlagNonFinite);
-    a.out[idx] = v;
 }
 
 // prange_kernel (stage_generic.cuh) on 2-D grids.
 template <int SCHEME, typename R>
-__global__ void __launch_bounds__(256) prange_plane_kernel(StageArgs<R> a, StepChoice ch)
+__global__ void __launch_bounds__(256) prange_plane_kernel(StageArgs<R> a, PlaneConst<R> pc, StepChoice ch)
 {
     stage_wait();
     stage_release();
@@ -205,7 +239,7 @@ __global__ void __launch_bounds__(256) prange_plane_kernel(StageArgs<R> a, StepC
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             R am, ap;
-            plane_derivs<SCHEME>(u[k], Num<R>::eps_floor(a.inv_dx[k]), am, ap);
+            plane_derivs<SCHEME>(u[k], pc.floor_[k], am, ap);
             m[k] = rmax(rabs(am), rabs(ap)) * a.inv_dx[k];
         }
     }

@@ -23,10 +23,10 @@ namespace lsp {
 // agree to rounding anyway.
 template <typename R> struct Num;
 template <> struct Num<float> {
-    static __device__ __forceinline__ float eps_floor(float /*inv_dx*/) { return 1e-18f; }
+    static __host__ __device__ __forceinline__ float eps_floor(float /*inv_dx*/) { return 1e-18f; }
 };
 template <> struct Num<double> {
-    static __device__ __forceinline__ double eps_floor(double inv_dx)
+    static __host__ __device__ __forceinline__ double eps_floor(double inv_dx)
     {
         return 1e-99 / (inv_dx * inv_dx);
     }
