@@ -772,7 +772,7 @@ lsp_status lsp_hj_solve(lsp_grid* g, const lsp_solve_opts* o, void* phi, const v
     if (!g->alpha_state) {
         // Alpha, and with it the step, comes from phi: the device chooses
         // each step (finish_prange) and the host enqueues steps ahead of it,
-        // as many as the last one's length suggests and a few more; steps
+        // as many as the last one's length suggests (steps_ahead); steps
         // past the last leave the fields alone.  One read-back per batch
         // instead of one per step, and no memset per stage (257 x 193 WENO5
         // RK3 FP32, 12 steps: 714 -> 606 us).
@@ -800,8 +800,7 @@ lsp_status lsp_hj_solve(lsp_grid* g, const lsp_solve_opts* o, void* phi, const v
             if (e) return cuda_fail(e, "synchronize");
             if (c.stop_at) break;
             if (!(c.dt > 0.0)) return fail(LSP_EINVAL, "non-positive CFL step");
-            const double left = std::ceil((t_stop - c.t) / c.dt);
-            batch = (int)std::fmin(256.0, std::fmax(1.0, left) + 1.0 + std::floor(left / 16.0));
+            batch = lsp::steps_ahead((t_stop - c.t) / c.dt);
         }
         sts.steps = (int64_t)c.steps;
         sts.stages = sts.steps * o->rk_order;
