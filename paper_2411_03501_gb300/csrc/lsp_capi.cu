@@ -17,6 +17,7 @@
 #include "stage_generic.cuh"
 #include "stage_march.cuh"
 #include "stage_tiled.cuh"
+#include "tile_rules.h"
 
 struct lsp_grid {
     int ndim = 0;
@@ -204,63 +205,13 @@ void march_tiles(const lsp_grid* g, int scheme, std::vector<lsp::Tile>* out)
     for (const auto& c : got) out->push_back(c.second);
 }
 
-// Tile of the paired shared-face WENO5 kernel (stage_pair.cuh) on a 3-D grid:
-// the lowest estimate
-//   (ch / 2 + 0.1) (CTAs per SM x warps (1 + 0.1 frame / tile) + 5 waves)
-// in units of one warp's issue time per pair of planes, over tiles of 64 to
-// 256 threads that split both axes evenly and a few even chunk lengths, for 3
-// CTAs of 256 threads per SM.  Fitted to sweeps of tile and chunk on seven
-// grids; us per stage, 16 x 16 tiles in chunks for three waves before, this
-// rule, the best of the sweep: 41^3 9.7, 6.1, 6.0; 25x60x90 9.9, 7.2, 7.2;
-// 97x113x85 25.4, 22.8, 22.2; 30x150x45 9.9, 8.5, 8.5; 129^3 46.2, 40.4,
-// 40.4; 201^3 123.5, 124.0, 123.0; 60x61x62 9.9, 9.9, 9.5.
-lsp::Tile pair_tile(const lsp_grid* g)
-{
-    lsp::Tile best{0, 0, 0, 3, 2};
-    if (g->ndim != 3) return best;
-    const int nS = g->n[0], nA = g->n[1], nB = g->n[2], G = 3;
-    const long long sms = lsp::sm_count();
-    double best_cost = INFINITY;
-    for (int kb = 1; kb <= nB; ++kb) {
-        const int tb = (nB + kb - 1) / kb;
-        if (tb < 8) break;
-        if (tb > 64 || (kb > 1 && tb == (nB + kb - 2) / (kb - 1))) continue;
-        for (int ka = (nA * tb + 255) / 256; ka <= nA; ++ka) {
-            const int ta = (nA + ka - 1) / ka;
-            if (ta < 4 || tb * ta < 64) break;
-            if (tb * ta > 256 || (ka > 1 && ta == (nA + ka - 2) / (ka - 1))) continue;
-            lsp::Tile t{tb, ta, 2, 3, 2};
-            if (!lsp::tile_valid(3, LSP_WENO5, t, g->n)) continue;
-            const int warps = (tb * ta + 31) / 32;
-            const int resident = std::min(65536 / (80 * 32 * warps), 32);
-            const double weight = warps * (1.0 + 0.1 * 2 * G * (tb + ta) / (tb * ta));
-            const long long plane_ctas = (long long)((nB + tb - 1) / tb) * ((nA + ta - 1) / ta);
-            for (const int ch : {2, 4, 6, 8, 10, 12, 16, 20, 26, 34, 50, 66, 102}) {
-                if (ch > nS + 1) break;
-                const long long ctas = plane_ctas * ((nS + ch - 1) / ch);
-                const long long per_sm = (ctas + sms - 1) / sms;
-                const long long waves = (per_sm + resident - 1) / resident;
-                const double cost = (0.5 * ch + 0.1) * (per_sm * weight + 5.0 * waves);
-                if (cost < best_cost || (cost == best_cost && tb * ta > best.tb * best.ta)) {
-                    best_cost = cost;
-                    best = t;
-                    best.ch = ch;
-                }
-            }
-        }
-    }
-    return best;
-}
-
 // The tile used without lsp_set_tile / lsp_autotune.  WENO5 runs the paired
-// shared-face kernel, on 3-D grids with the tile of pair_tile, in 4-D on 16 x
-// 16 tiles, chunked so that the launch has about three waves of 3 CTAs per
-// SM, with an even chunk length (the pairs of planes).  ENO2/ENO3 with global coefficients run the register-marching
-// kernel (rockets 300^3: 165 us per stage against 388 for the scalar kernel's
-// 32 x 8 tiles, car4d 81^4: 438 against 860, 33 x 41 x 37 x 29: 21 against
-// 47); where no tile of it fits the grid, with local coefficients or the
-// clip, and for first order, the scalar kernel on 32 x 8 tiles, about two
-// waves of 2 CTAs per SM.
+// shared-face kernel, on 3-D grids with the tile of pair_rule where that is
+// estimated to be faster than 16 x 16 tiles.  ENO2/ENO3 with global
+// coefficients run the register-marching kernel (figures in stage_march.cuh);
+// where no tile of it fits the grid, with local coefficients or the clip, and
+// for first order, the scalar kernel on 32 x 8 tiles, about two waves of 2 CTAs
+// per SM.
 lsp::Tile default_tile(const lsp_grid* g, const lsp_solve_opts* o)
 {
     const int d = g->ndim, scheme = o->scheme;
@@ -268,22 +219,20 @@ lsp::Tile default_tile(const lsp_grid* g, const lsp_solve_opts* o)
         const lsp::Tile& t = g->march[scheme == LSP_ENO3];
         if (t.ch > 0) return t;
     }
-    const bool paired = scheme == LSP_WENO5;
-    if (paired && g->pair.ch > 0) return g->pair;
-    lsp::Tile t;
-    t.tb = paired ? 16 : 32;
-    t.ta = paired ? 16 : 8;
-    t.minb = 3;
-    t.pair = paired ? 2 : 0;
+    if (scheme == LSP_WENO5) {
+        if (g->pair.ch > 0) return g->pair;
+        const lsp::RuleTile q = lsp::pair_square_tile(d, g->n, lsp::sm_count());
+        return lsp::Tile{q.tb, q.ta, q.ch, 3, 2};
+    }
+    lsp::Tile t{32, 8, 0, 3, 0};
     const long long nplane = (long long)((g->n[d - 1] + t.tb - 1) / t.tb) *
                              ((g->n[d - 2] + t.ta - 1) / t.ta) * (d == 4 ? g->n[0] : 1);
-    const long long want = (paired ? 3LL * 3 : 2LL * 2) * lsp::sm_count();
+    const long long want = 2LL * 2 * lsp::sm_count();
     long long nch = (want + nplane - 1) / nplane;
     const int nS = g->n[d - 3];
     if (nch > nS / 4) nch = nS / 4;
     if (nch < 1) nch = 1;
     t.ch = (int)((nS + nch - 1) / nch);
-    if (paired && (t.ch & 1)) t.ch += 1;
     return t;
 }
 
@@ -636,7 +585,10 @@ lsp_status lsp_set_dynamics(lsp_grid* g, int dyn, const double* params, int npar
             march_tiles(g, scheme, &tiles);
             if (!tiles.empty()) g->march[scheme == LSP_ENO3] = tiles.front();
         }
-        g->pair = pair_tile(g);
+        if (g->ndim == 3) {
+            const lsp::RuleTile q = lsp::pair_rule(g->n, lsp::sm_count());
+            g->pair = lsp::Tile{q.tb, q.ta, q.ch, 3, 2};
+        }
     }
     for (int i = 0; i < LSP_NPARAM; ++i) g->prm[i] = i < need ? params[i] : 0.0;
     g->dyn = dyn;

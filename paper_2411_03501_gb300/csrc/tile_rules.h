@@ -1,0 +1,88 @@
+// tile_rules.h -- default tiles chosen by an estimate of a stage's time: host
+// arithmetic alone.
+#pragma once
+#include <algorithm>
+#include <cmath>
+
+namespace lsp {
+
+struct RuleTile {
+    int tb, ta, ch;  // ch = 0: no tile
+};
+
+// The 16 x 16 tile of the paired shared-face WENO5 kernel (stage_pair.cuh) in
+// chunks for about three waves of 3 CTAs per SM, of even length (its planes
+// are paired).  d = 3 or 4 axes.
+inline RuleTile pair_square_tile(int d, const int* n, long long sms)
+{
+    const long long nplane = (long long)((n[d - 1] + 15) / 16) * ((n[d - 2] + 15) / 16) * (d == 4 ? n[0] : 1);
+    const int nS = n[d - 3];
+    const long long nch = std::max(1LL, std::min((9 * sms + nplane - 1) / nplane, (long long)nS / 4));
+    const int ch = (int)((nS + nch - 1) / nch);
+    return {16, 16, ch + (ch & 1)};
+}
+
+// Estimated time of a stage of that kernel on a 3-D grid, in units of one
+// warp's issue time per pair of planes (80 ns):
+//   25 + sqrt(W^2 + L^2) + 0.5 k (ch / 2 + 0.75) warps'
+// with warps' = warps (1 + 0.29 frame / tile); W the warp pairs per SM, each
+// chunk 0.75 pairs more than its length; L the latency of the chain of
+// chunks, 20 per pair and wave of resident CTAs; the last term the tail of the
+// launch, half of the k CTAs an SM holds (3 of 256 threads).  Fitted to 5,200
+// timings on 150 random grids of 2,000 to 25 million nodes (root mean square
+// error 8 %).
+inline double pair_cost(const int* n, const RuleTile& t, long long sms)
+{
+    const int nS = n[0], nA = n[1], nB = n[2], G = 3;
+    const int warps = (t.tb * t.ta + 31) / 32;
+    const double resident = std::min(65536 / (80 * 32 * warps), 32);
+    const double unit = warps * (1.0 + 0.29 * 2 * G * (t.tb + t.ta) / (t.tb * t.ta));
+    const double columns = (double)((nB + t.tb - 1) / t.tb) * ((nA + t.ta - 1) / t.ta);
+    const double chunks = (nS + t.ch - 1) / t.ch, ctas = columns * chunks;
+    const double chunk = 0.5 * std::min(t.ch, nS) + 0.75;
+    const double k = std::min(std::ceil(ctas / sms), resident);
+    const double W = columns * (0.5 * nS + 0.75 * chunks) * unit / sms;
+    const double L = 20.0 * chunk * std::max(1.0, ctas / (sms * resident));
+    return 25.0 + std::sqrt(W * W + L * L) + 0.5 * k * chunk * unit;
+}
+
+// Tile of that kernel on a 3-D grid: the lowest estimate over tiles of 64 to
+// 256 threads that split both axes evenly and a few even chunk lengths, where
+// it is 10 % below the square tile's, else none (the square tile is used).
+// Against the square tile on 120 other random grids: geometric mean 0.77 of
+// its time, the slowest 1.014.  us per stage, square tile and this rule: 41^3
+// 9.7, 5.4; 97x113x85 25.4, 22.5; 129^3 46.2, 40.4; 201^3 (square) 123.6.  (An
+// estimate without the margin, and without the work of the chunks as such, was
+// up to 1.3 times slower than the square tile on 22 of 150 grids.)
+inline RuleTile pair_rule(const int* n, long long sms)
+{
+    const int nS = n[0], nA = n[1], nB = n[2], G = 3;
+    RuleTile best{0, 0, 0};
+    double best_cost = 0.0;
+    const auto even = [](int axis, int t) {  // t splits the axis evenly
+        const int k = (axis + t - 1) / t;
+        return (axis + k - 1) / k == t;
+    };
+    for (int tb = std::min(64, nB); tb >= 8; --tb) {
+        if (!even(nB, tb)) continue;
+        for (int ta = std::min(256 / tb, nA); ta >= 4 && tb * ta >= 64; --ta) {
+            if (!even(nA, ta) || (nA + ta - 1) / ta > 65535) continue;
+            // the haloed tile in 3 values per thread
+            if ((ta + 2 * G) * (tb + 2 * G) > 3 * ta * tb) continue;
+            for (const int ch : {2, 4, 6, 8, 10, 12, 16, 20, 26, 34, 50, 66, 102}) {
+                if (ch > nS + 1) break;
+                const RuleTile t{tb, ta, ch};
+                if ((nS + ch - 1) / ch > 65535) continue;
+                const double c = pair_cost(n, t, sms);
+                if (best.ch == 0 || c < best_cost) {
+                    best = t;
+                    best_cost = c;
+                }
+            }
+        }
+    }
+    if (best.ch && pair_cost(n, pair_square_tile(3, n, sms), sms) <= 1.1 * best_cost) best.ch = 0;
+    return best;
+}
+
+}  // namespace lsp
