@@ -583,7 +583,12 @@ lsp_status lsp_set_dynamics(lsp_grid* g, int dyn, const double* params, int npar
         std::vector<lsp::Tile> tiles;
         for (const int scheme : {LSP_ENO2, LSP_ENO3}) {
             march_tiles(g, scheme, &tiles);
-            if (!tiles.empty()) g->march[scheme == LSP_ENO3] = tiles.front();
+            if (tiles.empty()) continue;
+            const lsp::Tile& t = tiles.front();
+            if (scheme == LSP_ENO3 && g->ndim == 4 &&
+                lsp::march_wasteful(g->n, {t.tb, t.ta, t.ch}, lsp::march_threads(t), lsp::sm_count()))
+                continue;
+            g->march[scheme == LSP_ENO3] = t;
         }
         if (g->ndim == 3) {
             const lsp::RuleTile q = lsp::pair_rule(g->n, lsp::sm_count());

@@ -85,4 +85,22 @@ inline RuleTile pair_rule(const int* n, long long sms)
     return best;
 }
 
+// Would the marching kernel's tile (stage_march.cuh) compute more than two
+// nodes per node of a 4-D grid, in more than one wave of CTAs?  Its tiles are
+// moved back from an axis' end, nodes under two of them computed twice, and a
+// chunk starts at the cost of two planes.  ENO3 with 7 rows (the shortest axis;
+// its frame allows tiles of 6 there) is then slower than the scalar kernel: 69
+// x 14 x 7 x 800 (2.01) 120 us per stage against 104, 7 x 7 x 7 x 3000 (2.5)
+// 40 against 34; 25 x 39 x 7 x 263 (2.24) 49.2, 49.6; 47 x 72 x 7 x 169 (1.996)
+// 89, 97.  A single wave is bound by latency, and the march is faster (7 x 53 x
+// 7 x 497, 2.4: 36 against 42).
+inline bool march_wasteful(const int* n, const RuleTile& t, int threads, long long sms)
+{
+    const auto up = [](int a, int b) { return (a + b - 1) / b; };
+    const int ch = std::min(t.ch, n[1]);
+    const double computed = (double)up(n[3], t.tb) * t.tb * up(n[2], t.ta) * t.ta * up(n[0], 2) * 2 * (ch + 2) / ch;
+    const double ctas = (double)up(n[3], t.tb) * up(n[2], t.ta) * up(n[0], 2) * up(n[1], t.ch);
+    return computed > 2.0 * n[3] * n[2] * n[0] && ctas * threads > 512.0 * sms;
+}
+
 }  // namespace lsp

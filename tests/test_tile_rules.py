@@ -17,6 +17,10 @@ extern "C" void rule(const int* n, long long sms, int* out)
     const lsp::RuleTile t = lsp::pair_rule(n, sms), q = lsp::pair_square_tile(3, n, sms);
     out[0] = t.tb; out[1] = t.ta; out[2] = t.ch; out[3] = q.ch;
 }
+extern "C" int wasteful(const int* n, int tb, int ta, int ch, int threads, long long sms)
+{
+    return lsp::march_wasteful(n, {tb, ta, ch}, threads, sms);
+}
 """
 
 
@@ -32,6 +36,7 @@ def rule(tmp_path_factory):
         out = (ctypes.c_int * 4)()
         lib.rule((ctypes.c_int * 3)(*n), ctypes.c_longlong(sms), out)
         return tuple(out[:3]), (16, 16, out[3])
+    call.lib = lib
     return call
 
 
@@ -68,3 +73,14 @@ def test_tiles_can_be_launched(rule):
         assert -(-n[1] // ta) <= 65535 and -(-n[0] // ch) <= 65535
     # chosen when a grid gets its dynamics: microseconds, whatever the axes
     assert (time.perf_counter() - t0) / len(grids) < 2e-3
+
+
+@pytest.mark.parametrize("n,tile,wasteful", [([69, 14, 7, 800], (45, 6, 14, 160), True),
+                                             ([7, 7, 7, 3000], (45, 6, 7, 160), True),
+                                             ([7, 53, 7, 497], (46, 6, 11, 160), False),
+                                             ([47, 72, 7, 169], (34, 6, 15, 128), False),
+                                             ([81, 81, 81, 81], (41, 12, 27, 256), False)])
+def test_march_tiles_that_compute_most_nodes_twice(rule, n, tile, wasteful):
+    """Slower than the scalar kernel where timed, and the ones next to them
+    that are faster."""
+    assert bool(rule.lib.wasteful((ctypes.c_int * 4)(*n), *tile, ctypes.c_longlong(152))) == wasteful
