@@ -36,12 +36,17 @@ inline BatchTiling batch_tiling(int ndim, const int* n, int shape, int chunk)
     return t;
 }
 
-// Planes of tiles a stage of this problem has.
-inline double batch_planes(int ndim, const int* n, int shape)
-{
-    const BatchTiling t = batch_tiling(ndim, n, shape, 1);
-    return (double)t.blocks;
-}
+// The work of a stage of the batch: planes of tiles, and the longest column of
+// planes.
+struct BatchWork {
+    double planes = 0.0;
+    int longest = 1;
+    void add(int ndim, const int* n, int shape)
+    {
+        planes += (double)batch_tiling(ndim, n, shape, 1).blocks;
+        if (ndim >= 3) longest = std::max(longest, n[ndim - 3]);
+    }
+};
 
 // Planes per CTA when opts->batch_chunk is 0.  A stage of the whole batch has
 // x = planes / (3 CTAs x SMs) planes for each resident CTA: with
@@ -57,9 +62,16 @@ inline double batch_planes(int ndim, const int* n, int shape)
 //   4 at 0.4 size, x = 1: 4 planes 0.31, 1.06 (4: 0.34, 1.09)
 //   96 problems, x = 390: 128 planes 8.97 (32: 9.25, 64: 9.29, 128: 9.89)
 // which 5 + 0.31 x (persistent) and 4 + 0.2 x (graph) meet within 3 %.
-inline int batch_auto_chunk(double planes, int sms, bool persistent)
+// Whole columns stay where no column is longer than x: they fill the device
+// evenly as they are (263 problems of 9^3 on 64 x 4 tiles 29 % faster whole,
+// 146 of 27 x 26 x 24 on 16 x 16 9 %); up to 24 planes, where a start weighs
+// more, from 0.6 of the longest on (graph form: 368 of 12^3, 130 of 20 x 21 x
+// 22 on 32 x 8, 14 %).  Over 250 random batches of 1 to 400 problems: 0.49
+// (persistent) and 0.53 (graph) of the time of whole columns, none above 1.04.
+inline int batch_auto_chunk(const BatchWork& w, int sms, bool persistent)
 {
-    const double x = planes / (3.0 * sms);
+    const double x = w.planes / (3.0 * sms);
+    if (x >= (w.longest <= 24 ? 0.6 : 1.0) * w.longest) return kBatchMaxPlanes;
     const double c = persistent ? 5.0 + 0.31 * x : 4.0 + 0.2 * x;
     return c >= kBatchMaxPlanes ? kBatchMaxPlanes : std::max(kBatchMinPlanes, (int)c / 2 * 2);
 }

@@ -1160,13 +1160,12 @@ void batch_geometry(int nprob, lsp_grid* const* grids, const lsp_solve_opts* o,
                     bool any_shape = false)
 {
     const bool local = o->diss != LSP_DISS_GLF || o->varform;
-    double planes = 0.0;
+    lsp::BatchWork work;
     for (int i = 0; i < nprob; ++i)
-        planes += lsp::batch_planes(grids[i]->ndim, grids[i]->n,
-                                    lsp::batch_shape(o->batch_tiles, grids[i]->ndim, local));
+        work.add(grids[i]->ndim, grids[i]->n, lsp::batch_shape(o->batch_tiles, grids[i]->ndim, local));
     const int chunk = o->batch_chunk > 0
                           ? o->batch_chunk
-                          : lsp::batch_auto_chunk(planes, lsp::sm_count(), o->batch_persistent != 0);
+                          : lsp::batch_auto_chunk(work, lsp::sm_count(), o->batch_persistent != 0);
     plan.resize(nprob);
     size_t fields = 0;
     long long blocks = 0;

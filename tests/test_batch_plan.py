@@ -22,9 +22,9 @@ extern "C" long long sized(int np, const int* nd, const int (*n)[4], int chunk)
 extern "C" long long needed(int np, const int* nd, const int (*n)[4], int tiles, int chunk,
                             int persistent, int local, int sms)
 {
-    double planes = 0;
-    for (int i = 0; i < np; ++i) planes += batch_planes(nd[i], n[i], batch_shape(tiles, nd[i], local));
-    if (chunk <= 0) chunk = batch_auto_chunk(planes, sms, persistent);
+    BatchWork w;
+    for (int i = 0; i < np; ++i) w.add(nd[i], n[i], batch_shape(tiles, nd[i], local));
+    if (chunk <= 0) chunk = batch_auto_chunk(w, sms, persistent);
     long long b = 0;
     for (int i = 0; i < np; ++i) b += batch_tiling(nd[i], n[i], batch_shape(tiles, nd[i], local), chunk).blocks;
     return b;
@@ -84,3 +84,22 @@ def test_chunks_by_work_stay_in_their_range(plan):
     _, needed = plan
     assert needed([[64, 16, 16]], 0, 0, 0, 0, 152) == 16
     assert needed([[128, 16, 16]] * 4000, 0, 0, 1, 0, 152) == 4000
+
+
+@pytest.mark.parametrize("n,count,shape,persistent", [([9, 9, 9], 263, 2, 1), ([12, 12, 11], 231, 2, 1),
+                                                      ([15, 15, 15], 200, 2, 0), ([12, 12, 12], 368, 0, 0), ([20, 21, 22], 130, 1, 0),
+                                                      ([27, 26, 24], 146, 0, 1), ([42, 45, 41], 103, 0, 1)])
+def test_columns_that_fill_the_device_stay_whole(plan, n, count, shape, persistent):
+    """Timed 8 to 29 % faster than in chunks."""
+    _, needed = plan
+    tiles = shape << 2
+    whole = needed([n] * count, tiles, 128, persistent, 0, 152)
+    assert needed([n] * count, tiles, 0, persistent, 0, 152) == whole
+
+
+def test_uneven_batches_are_cut(plan):
+    """A few problems, or one long column among short ones."""
+    _, needed = plan
+    for grids in ([[129, 129, 129]], [[20 + 20 * i] * 3 for i in range(6)], [[15, 15, 15]] * 60 + [[200, 40, 40]]):
+        for persistent in (0, 1):
+            assert needed(grids, 0, 0, persistent, 0, 152) > 1.5 * needed(grids, 0, 200, persistent, 0, 152)
