@@ -23,7 +23,6 @@ struct ShapeDev {
     unsigned n[LSP_MAXD], m[LSP_MAXD];
     int l[LSP_MAXD];
     unsigned ignore, npts;
-    int kind;
 };
 
 // floor(x / n) for 0 <= x < 2^31 by a multiply-high and a shift (Granlund and
@@ -52,34 +51,31 @@ struct ShapePart {
     R q, in;
 };
 
-template <typename R>
+template <int KIND, typename R>
 __device__ __forceinline__ void shape_axis(const ShapeDev<R>& s, int k, R x, ShapePart<R>& p)
 {
     if ((s.ignore >> k) & 1u) return;
-    if (s.kind == SHAPE_SPHERE) {
+    if constexpr (KIND == SHAPE_SPHERE) {
         p.q += (x - s.c[k]) * (x - s.c[k]);
-    } else if (s.kind == SHAPE_BOX) {
+    } else if constexpr (KIND == SHAPE_BOX) {
         const R e = rmax(s.c[k] - x, x - s.d[k]);  // > 0 outside this slab
         if (e > R(0)) p.q += e * e;
         p.in = rmax(p.in, e);
-    } else if (s.kind == SHAPE_QUADRIC) {
+    } else if constexpr (KIND == SHAPE_QUADRIC) {
         p.q += s.d[k] * (x - s.c[k]) * (x - s.c[k]);
     } else {
         p.q += s.d[k] * (x - s.c[k]);
     }
 }
 
-template <int NDIM, typename R>
+template <int KIND, typename R>
 __device__ __forceinline__ R shape_finish(const ShapeDev<R>& s, const ShapePart<R>& p)
 {
-    if (s.kind == SHAPE_SPHERE) return real_sqrt(p.q) - s.r;             // |x - c| - r
-    if (s.kind == SHAPE_BOX) return p.q > R(0) ? real_sqrt(p.q) : p.in;  // exact distance to [c, d]
-    if (s.kind == SHAPE_QUADRIC) return p.q - s.r;  // sum_k w_k (x_k - c_k)^2 - offset
-    R nn = R(0);  // half space {n . (x - p) <= 0}: n . (x - p) / |n|
-#pragma unroll
-    for (int k = 0; k < NDIM; ++k)
-        if (!((s.ignore >> k) & 1u)) nn += s.d[k] * s.d[k];
-    return p.q / real_sqrt(nn);
+    if constexpr (KIND == SHAPE_SPHERE) return real_sqrt(p.q) - s.r;  // |x - c| - r
+    // exact distance to [c, d]
+    else if constexpr (KIND == SHAPE_BOX) return p.q > R(0) ? real_sqrt(p.q) : p.in;
+    else if constexpr (KIND == SHAPE_QUADRIC) return p.q - s.r;  // sum_k w_k (x_k - c_k)^2 - offset
+    else return p.q / s.r;  // half space {n . (x - p) <= 0}: n . (x - p) / |n|, r = |n|
 }
 
 // 16 bytes of consecutive values
@@ -88,58 +84,68 @@ struct alignas(V * sizeof(R)) Vec {
     R v[V];
 };
 
-// V consecutive nodes per thread (V values fill 16 bytes; 1 for a field that
-// is not 16-byte aligned): one index split by the axis lengths (the fastest
-// axis last), one store and, within a row, one pass over the other axes per V
-// nodes.  Coordinates lo + index * dx as the stage kernels compute them.
-// Dimensions are a template parameter, so everything stays in registers; the
-// host checks npts < 2^31 (32-bit index arithmetic).  Bound by the writes and
-// the launches: cylinder, box and their union at 201^3 FP32 49.6 us with one
-// node per thread and store, 41.2 us now (162 MB).
-template <int NDIM, typename R, int V>
+// V consecutive nodes per thread and round (V values fill 16 bytes; 1 for a
+// field that is not 16-byte aligned, or small: shape_vector_nodes): one index split
+// by the axis lengths (the fastest axis last), one store and, within a row,
+// one pass over the other axes per V nodes.  Coordinates lo + index * dx as
+// the stage kernels compute them.  Dimensions and the primitive are template
+// parameters, so everything stays in registers; the host checks npts < 2^31
+// (32-bit index arithmetic).  Bound by the writes and the launches in FP32 and
+// by the FP64 pipe in FP64.  A launch has at most 16 blocks per SM, in a
+// grid-stride loop: a block for every 256 threads' nodes is bound by the rate
+// at which blocks start.  us per call, back to back: one node per thread and
+// round with the primitive chosen in the kernel; V nodes in one pass of blocks;
+// this.  201^3 FP32 sphere 16.7, 16.5, 12.3; quadric 14.5, 18.6, 10.3; half
+// space 18.7, 22.8, 12.2; unaligned sphere 16.6, 22.8, 14.7; 400 x 401 x 402
+// half space 123, 148, 60; 201^3 FP64 half space (the norm from the host) 460,
+// 436, 256.  Cylinder, box and their union at 201^3 FP32: 49.6, 41.1, 35.6.
+template <int NDIM, int KIND, typename R, int V>
 __global__ void __launch_bounds__(256) shape_kernel(ShapeDev<R> s, R* out)
 {
-    const unsigned i0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
-    if (i0 >= s.npts) return;
-    Vec<R, V> w;
-    ShapePart<R> row;
-    unsigned c = 0, end = 0;  // fastest index of the next node, end of its row
+    for (unsigned i0 = (blockIdx.x * blockDim.x + threadIdx.x) * V; i0 < s.npts;
+         i0 += gridDim.x * blockDim.x * V) {
+        Vec<R, V> w;
+        ShapePart<R> row;
+        unsigned c = 0, end = 0;  // fastest index of the next node, end of its row
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-        if (v == 0 || c == end) {  // first node, or first of the next row
-            row.q = R(0);
-            row.in = R(-INFINITY);
-            unsigned r = i0 + v;
-            unsigned idx[NDIM];
+        for (int v = 0; v < V; ++v) {
+            if (v == 0 || c == end) {  // first node, or first of the next row
+                row.q = R(0);
+                row.in = R(-INFINITY);
+                unsigned r = i0 + v;
+                unsigned idx[NDIM];
 #pragma unroll
-            for (int k = NDIM - 1; k > 0; --k) {
-                const unsigned q = div_invariant(r, s.m[k], s.l[k]);
-                idx[k] = r - q * s.n[k];
-                r = q;
+                for (int k = NDIM - 1; k > 0; --k) {
+                    const unsigned q = div_invariant(r, s.m[k], s.l[k]);
+                    idx[k] = r - q * s.n[k];
+                    r = q;
+                }
+                idx[0] = r;
+#pragma unroll
+                for (int k = 0; k < NDIM - 1; ++k)
+                    shape_axis<KIND>(s, k, rfma(R(idx[k]), s.h[k], s.lo[k]), row);
+                c = idx[NDIM - 1];
+                end = s.n[NDIM - 1];
             }
-            idx[0] = r;
-#pragma unroll
-            for (int k = 0; k < NDIM - 1; ++k)
-                shape_axis(s, k, rfma(R(idx[k]), s.h[k], s.lo[k]), row);
-            c = idx[NDIM - 1];
-            end = s.n[NDIM - 1];
+            ShapePart<R> p = row;
+            shape_axis<KIND>(s, NDIM - 1, rfma(R(c), s.h[NDIM - 1], s.lo[NDIM - 1]), p);
+            w.v[v] = shape_finish<KIND>(s, p);
+            ++c;
         }
-        ShapePart<R> p = row;
-        shape_axis(s, NDIM - 1, rfma(R(c), s.h[NDIM - 1], s.lo[NDIM - 1]), p);
-        w.v[v] = shape_finish<NDIM>(s, p);
-        ++c;
-    }
-    if (i0 + V <= s.npts) {
-        *reinterpret_cast<Vec<R, V>*>(out + i0) = w;
-    } else {
+        if (i0 + V <= s.npts) {
+            *reinterpret_cast<Vec<R, V>*>(out + i0) = w;
+        } else {
 #pragma unroll
-        for (int v = 0; v < V; ++v)
-            if (i0 + v < s.npts) out[i0 + v] = w.v[v];
+            for (int v = 0; v < V; ++v)
+                if (i0 + v < s.npts) out[i0 + v] = w.v[v];
+        }
     }
 }
 
 // union min(a, b), intersection max(a, b), complement -a, difference
-// max(a, -b) (Sec. III-D), V consecutive values per thread
+// max(a, -b) (Sec. III-D), V consecutive values per thread and round, blocks
+// as for shape_kernel (union of two 201^3 FP32 fields, forms as above: 18.6,
+// 12.5, 10.6 us; unaligned 14.5, 28.9, 14.5)
 template <typename R>
 __device__ __forceinline__ R shape_op_value(int op, R u, R b)
 {
@@ -155,46 +161,61 @@ template <typename R, int V>
 __global__ void __launch_bounds__(256) shape_op_kernel(int op, const R* a, const R* b, R* out,
                                                        unsigned n)
 {
-    const unsigned i = (blockIdx.x * blockDim.x + threadIdx.x) * V;
-    if (i >= n) return;
-    if (i + V <= n) {
-        const Vec<R, V> u = *reinterpret_cast<const Vec<R, V>*>(a + i);
-        Vec<R, V> w = u;
-        if (op != LSP_SHAPE_COMPLEMENT) w = *reinterpret_cast<const Vec<R, V>*>(b + i);
+    for (unsigned i = (blockIdx.x * blockDim.x + threadIdx.x) * V; i < n; i += gridDim.x * blockDim.x * V) {
+        if (i + V <= n) {
+            const Vec<R, V> u = *reinterpret_cast<const Vec<R, V>*>(a + i);
+            Vec<R, V> w = u;
+            if (op != LSP_SHAPE_COMPLEMENT) w = *reinterpret_cast<const Vec<R, V>*>(b + i);
 #pragma unroll
-        for (int v = 0; v < V; ++v) w.v[v] = shape_op_value(op, u.v[v], w.v[v]);
-        *reinterpret_cast<Vec<R, V>*>(out + i) = w;
-    } else {
-        for (unsigned j = i; j < n; ++j)
-            out[j] = shape_op_value(op, a[j], op == LSP_SHAPE_COMPLEMENT ? R(0) : b[j]);
+            for (int v = 0; v < V; ++v) w.v[v] = shape_op_value(op, u.v[v], w.v[v]);
+            *reinterpret_cast<Vec<R, V>*>(out + i) = w;
+        } else {
+            for (unsigned j = i; j < n; ++j)
+                out[j] = shape_op_value(op, a[j], op == LSP_SHAPE_COMPLEMENT ? R(0) : b[j]);
+        }
     }
 }
 
 static unsigned shape_blocks(long long n, int v)
 {
-    const long long t = (n + v - 1) / v;
-    return (unsigned)((t + 255) / 256);
+    const long long t = (n + v - 1) / v, b = (t + 255) / 256, cap = 16LL * sm_count();
+    return (unsigned)(b < cap ? b : cap);
 }
+// Fewest nodes for V consecutive ones per thread: two blocks per SM.  Below,
+// the chain of V nodes in one thread is longer than what it saves.
+static unsigned shape_vector_nodes(int v) { return 512u * v * sm_count(); }
 static bool vec_aligned(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-template <typename R, int V>
+template <int KIND, typename R, int V>
 static cudaError_t shape_launch(int ndim, const ShapeDev<R>& d, R* out, cudaStream_t st)
 {
     const unsigned nb = shape_blocks(d.npts, V);
     switch (ndim) {
-    case 1: shape_kernel<1, R, V><<<nb, 256, 0, st>>>(d, out); break;
-    case 2: shape_kernel<2, R, V><<<nb, 256, 0, st>>>(d, out); break;
-    case 3: shape_kernel<3, R, V><<<nb, 256, 0, st>>>(d, out); break;
-    case 4: shape_kernel<4, R, V><<<nb, 256, 0, st>>>(d, out); break;
+    case 1: shape_kernel<1, KIND, R, V><<<nb, 256, 0, st>>>(d, out); break;
+    case 2: shape_kernel<2, KIND, R, V><<<nb, 256, 0, st>>>(d, out); break;
+    case 3: shape_kernel<3, KIND, R, V><<<nb, 256, 0, st>>>(d, out); break;
+    case 4: shape_kernel<4, KIND, R, V><<<nb, 256, 0, st>>>(d, out); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
+}
+
+template <typename R, int V>
+static cudaError_t shape_kind(int kind, int ndim, const ShapeDev<R>& d, R* out, cudaStream_t st)
+{
+    switch (kind) {
+    case SHAPE_SPHERE: return shape_launch<SHAPE_SPHERE, R, V>(ndim, d, out, st);
+    case SHAPE_BOX: return shape_launch<SHAPE_BOX, R, V>(ndim, d, out, st);
+    case SHAPE_QUADRIC: return shape_launch<SHAPE_QUADRIC, R, V>(ndim, d, out, st);
+    default: return shape_launch<SHAPE_HALFSPACE, R, V>(ndim, d, out, st);
+    }
 }
 
 template <typename R>
 static cudaError_t launch_shape_t(const ShapeGeom& g, const ShapeArgs& s, R* out, cudaStream_t st)
 {
     ShapeDev<R> d;
+    R nn = R(0);  // |n|^2 of a half space
     for (int k = 0; k < LSP_MAXD; ++k) {
         const bool used = k < g.ndim;
         d.lo[k] = used ? R(g.lo[k]) : R(0);
@@ -203,13 +224,14 @@ static cudaError_t launch_shape_t(const ShapeGeom& g, const ShapeArgs& s, R* out
         d.d[k] = used ? R(s.d[k]) : R(0);
         d.n[k] = used ? (unsigned)g.n[k] : 1u;
         division_multiplier(d.n[k], &d.m[k], &d.l[k]);
+        if (used && !((s.ignore >> k) & 1u)) nn = std::fma(d.d[k], d.d[k], nn);
     }
-    d.r = R(s.r);
+    d.r = s.kind == SHAPE_HALFSPACE ? std::sqrt(nn) : R(s.r);
     d.ignore = s.ignore;
     d.npts = (unsigned)g.npts;
-    d.kind = s.kind;
     constexpr int V = 16 / sizeof(R);
-    return vec_aligned(out) ? shape_launch<R, V>(g.ndim, d, out, st) : shape_launch<R, 1>(g.ndim, d, out, st);
+    return vec_aligned(out) && d.npts >= shape_vector_nodes(V) ? shape_kind<R, V>(s.kind, g.ndim, d, out, st)
+                                                              : shape_kind<R, 1>(s.kind, g.ndim, d, out, st);
 }
 
 cudaError_t launch_shape(const ShapeGeom& g, const ShapeArgs& s, int dtype, void* out,
@@ -223,7 +245,8 @@ template <typename R>
 static cudaError_t launch_op_t(int op, const R* a, const R* b, R* out, long long n, cudaStream_t st)
 {
     constexpr int V = 16 / sizeof(R);
-    if (vec_aligned(a) && (op == LSP_SHAPE_COMPLEMENT || vec_aligned(b)) && vec_aligned(out))
+    if (n >= shape_vector_nodes(V) && vec_aligned(a) && (op == LSP_SHAPE_COMPLEMENT || vec_aligned(b)) &&
+        vec_aligned(out))
         shape_op_kernel<R, V><<<shape_blocks(n, V), 256, 0, st>>>(op, a, b, out, (unsigned)n);
     else
         shape_op_kernel<R, 1><<<shape_blocks(n, 1), 256, 0, st>>>(op, a, b, out, (unsigned)n);
