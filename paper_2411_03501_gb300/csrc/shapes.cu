@@ -146,32 +146,31 @@ __global__ void __launch_bounds__(256) shape_kernel(ShapeDev<R> s, R* out)
 // max(a, -b) (Sec. III-D), V consecutive values per thread and round, blocks
 // as for shape_kernel (union of two 201^3 FP32 fields, forms as above: 18.6,
 // 12.5, 10.6 us; unaligned 14.5, 28.9, 14.5)
-template <typename R>
-__device__ __forceinline__ R shape_op_value(int op, R u, R b)
+template <int OP, typename R>
+__device__ __forceinline__ R shape_op_value(R u, R b)
 {
-    switch (op) {
-    case LSP_SHAPE_UNION: return fmin(u, b);
-    case LSP_SHAPE_INTERSECT: return fmax(u, b);
-    case LSP_SHAPE_COMPLEMENT: return -u;
-    default: return fmax(u, -b);
-    }
+    if constexpr (OP == LSP_SHAPE_UNION) return fmin(u, b);
+    else if constexpr (OP == LSP_SHAPE_INTERSECT) return fmax(u, b);
+    else if constexpr (OP == LSP_SHAPE_COMPLEMENT) return -u;
+    else return fmax(u, -b);
 }
 
-template <typename R, int V>
-__global__ void __launch_bounds__(256) shape_op_kernel(int op, const R* a, const R* b, R* out,
-                                                       unsigned n)
+template <int OP, typename R, int V>
+__global__ void __launch_bounds__(256) shape_op_kernel(const R* a, const R* b, R* out, unsigned n)
 {
     for (unsigned i = (blockIdx.x * blockDim.x + threadIdx.x) * V; i < n; i += gridDim.x * blockDim.x * V) {
         if (i + V <= n) {
             const Vec<R, V> u = *reinterpret_cast<const Vec<R, V>*>(a + i);
             Vec<R, V> w = u;
-            if (op != LSP_SHAPE_COMPLEMENT) w = *reinterpret_cast<const Vec<R, V>*>(b + i);
+            if constexpr (OP != LSP_SHAPE_COMPLEMENT) w = *reinterpret_cast<const Vec<R, V>*>(b + i);
 #pragma unroll
-            for (int v = 0; v < V; ++v) w.v[v] = shape_op_value(op, u.v[v], w.v[v]);
+            for (int v = 0; v < V; ++v) w.v[v] = shape_op_value<OP>(u.v[v], w.v[v]);
             *reinterpret_cast<Vec<R, V>*>(out + i) = w;
         } else {
-            for (unsigned j = i; j < n; ++j)
-                out[j] = shape_op_value(op, a[j], op == LSP_SHAPE_COMPLEMENT ? R(0) : b[j]);
+            for (unsigned j = i; j < n; ++j) {
+                if constexpr (OP == LSP_SHAPE_COMPLEMENT) out[j] = shape_op_value<OP>(a[j], R(0));
+                else out[j] = shape_op_value<OP>(a[j], b[j]);
+            }
         }
     }
 }
@@ -241,16 +240,27 @@ cudaError_t launch_shape(const ShapeGeom& g, const ShapeArgs& s, int dtype, void
     return launch_shape_t<float>(g, s, (float*)out, st);
 }
 
+template <int OP, typename R>
+static cudaError_t op_launch(const R* a, const R* b, R* out, long long n, cudaStream_t st)
+{
+    constexpr int V = 16 / sizeof(R);
+    if (n >= shape_vector_nodes(V) && vec_aligned(a) && (OP == LSP_SHAPE_COMPLEMENT || vec_aligned(b)) &&
+        vec_aligned(out))
+        shape_op_kernel<OP, R, V><<<shape_blocks(n, V), 256, 0, st>>>(a, b, out, (unsigned)n);
+    else
+        shape_op_kernel<OP, R, 1><<<shape_blocks(n, 1), 256, 0, st>>>(a, b, out, (unsigned)n);
+    return cudaGetLastError();
+}
+
 template <typename R>
 static cudaError_t launch_op_t(int op, const R* a, const R* b, R* out, long long n, cudaStream_t st)
 {
-    constexpr int V = 16 / sizeof(R);
-    if (n >= shape_vector_nodes(V) && vec_aligned(a) && (op == LSP_SHAPE_COMPLEMENT || vec_aligned(b)) &&
-        vec_aligned(out))
-        shape_op_kernel<R, V><<<shape_blocks(n, V), 256, 0, st>>>(op, a, b, out, (unsigned)n);
-    else
-        shape_op_kernel<R, 1><<<shape_blocks(n, 1), 256, 0, st>>>(op, a, b, out, (unsigned)n);
-    return cudaGetLastError();
+    switch (op) {
+    case LSP_SHAPE_UNION: return op_launch<LSP_SHAPE_UNION>(a, b, out, n, st);
+    case LSP_SHAPE_INTERSECT: return op_launch<LSP_SHAPE_INTERSECT>(a, b, out, n, st);
+    case LSP_SHAPE_COMPLEMENT: return op_launch<LSP_SHAPE_COMPLEMENT>(a, b, out, n, st);
+    default: return op_launch<LSP_SHAPE_DIFFERENCE>(a, b, out, n, st);
+    }
 }
 
 cudaError_t launch_shape_op(int op, int dtype, const void* a, const void* b, void* out, long long n,
