@@ -13,8 +13,9 @@
 //  - FP64 maxima and the finiteness test run on the bits of the values in the
 //    integer pipe, the launch's constants come from the host (PlaneConst),
 //    and WENO5 divides once per side instead of four times.  Otherwise the
-//    operations and their order are the generic kernel's (ENO2 and ENO3 give
-//    its bits).
+//    operations and their order are the generic kernel's (first order, ENO2
+//    and ENO3 give its results to the rounding of products that the compiler
+//    fuses into sums).
 // Measured (GB300, us per stage of whole solves, generic kernel before):
 // 101 x 101 FP64 ENO2 8.7, 5.0; 127 x 93 FP64 WENO5 31.8, 13.6; 513 x 401
 // FP64 WENO5 176, 128 (the FP64 pipe); 301 x 177 FP32 WENO5 6.6, 3.9; 4096^2

@@ -27,3 +27,17 @@ def test_march_forms_equal_the_scalar_body(n, tile, scheme):
     dt = B.lsp_cfl_dt(P.grid, P.opts, 0.0, 1e9)
     assert P.solve(x, g, 0.0, 1.5 * dt)["steps"] == S.solve(y, g, 0.0, 1.5 * dt)["steps"] == 2
     assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("spec", [W.rockets(n=27)[0], W.air3d(nx=[37, 29, 45], scheme="eno3")[0], W.car4d(n=15)[0]],
+                         ids=["rockets", "air3d", "car4d"])
+def test_march_with_a_heading_equals_the_scalar_body(spec):
+    P, S = B.Problem(spec), B.Problem(spec)
+    assert P.tile()[4] == 6
+    S.set_tile(32, 8, 4, 3, 0)
+    x = torch.rand(spec["n"], device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    y, g = x.clone(), x + 0.05
+    dt = B.lsp_cfl_dt(P.grid, P.opts, 0.0, 1e9)
+    P.solve(x, g, 0.0, 3.5 * dt)
+    S.solve(y, g, 0.0, 3.5 * dt)
+    assert torch.equal(x, y)
