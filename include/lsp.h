@@ -302,7 +302,7 @@ lsp_status lsp_get_tile(const lsp_grid* grid, const lsp_solve_opts* opts, int* t
  * 1, 2; ENO2 and ENO3: pair 0, 1, plus the face-shared runs of pairs 3 and
  * 4 on 3 widths x 6 row counts x 7 chunk lengths and the 12 tiles of pair 6
  * with the lowest estimated cost), re-time the
- * six fastest over longer windows and keep the best in the grid handle
+ * six fastest and the default tile over longer windows and keep the best in the grid handle
  * (reported through tb/ta/ch/minb/pair, which may be NULL).  Waits for the
  * GPU.  For grids without a tiled kernel it selects the generic one (all
  * -1).  LSP_EUNSUPPORTED for QUADRATIC. */

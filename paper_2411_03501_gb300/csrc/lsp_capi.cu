@@ -970,7 +970,7 @@ lsp_status lsp_autotune(lsp_grid* g, const lsp_solve_opts* o, const void* phi, v
     // the fastest few of the first round, re-timed over longer windows
     constexpr int kFinal = 6;
     float top_ms[kFinal];
-    lsp::Tile top[kFinal];
+    lsp::Tile top[kFinal + 1];
     int ntop = 0;
     const double dt = cfl_dt_host(g, o->cfl, 0.0, INFINITY);
     auto run_once = [&]() -> lsp_status {
@@ -1056,6 +1056,11 @@ lsp_status lsp_autotune(lsp_grid* g, const lsp_solve_opts* o, const void* phi, v
         }
         if (s) break;
     }
+    // the tile used without tuning is always a finalist: it is fitted to the
+    // grid by rules of its own (60 x 9 x 300 WENO5 9.0 us per stage, the best of
+    // the shapes above 11.5)
+    const lsp::Tile plain = default_tile(g, o);
+    if (lsp::tile_valid(d, o->scheme, plain, g->n)) top[ntop++] = plain;
     // second round: each finalist timed as the best of 3 windows of 3
     // back-to-back runs (single runs of ~0.1-1 ms differ by a few %)
     for (int i = 0; i < ntop && !s; ++i) {
