@@ -135,7 +135,8 @@ def launch_accounting(spec, tile, stats) -> tuple[int, float, float, bool]:
 
 KERNEL_SOURCES = ["stencil.cuh", "stage_tiled.cuh", "stage_tiled.inl", "stage_generic.cuh",
                   "pair2.cuh", "stage_pair.cuh", "stage_run.cuh", "stage_run.inl",
-                  "stage_march.cuh", "stage_march.inl"]
+                  "stage_march.cuh", "stage_march.inl", "stage_plane.cuh",
+                  "lsp_internal.h"]
 
 
 def kernel_hash() -> str:

@@ -5,9 +5,11 @@
 
 namespace lsp {
 
-// Launch of a kernel that begins with stage_begin() (lsp_internal.h): its CTAs
+// Launch of a kernel that calls stage_wait() and then stage_release()
+// (lsp_internal.h) before it touches a field or the control block: its CTAs
 // may start while the previous kernel of the stream is still running, once
-// every CTA of that one has started.
+// every CTA of that one has released or finished.  A kernel launched this way
+// without the wait would race with the previous stage.
 template <typename... P, typename... A>
 cudaError_t launch_dependent(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                              A... args)

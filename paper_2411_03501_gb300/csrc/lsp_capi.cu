@@ -136,9 +136,11 @@ double cfl_dt_host(const lsp_grid* g, double cfl, double t, double t_final)
 }
 
 // Longest chunk the marching kernel gets by default on 4-D grids, where longer
-// ones are slower than the estimate says (car4d 81^4, 41 x 12 tiles: 424 us
-// per stage with 21 planes, 434 with 27, 490 with 41, 485 with 81): the CTAs of
-// a wave drift apart and the slabs they share leave the caches.
+// ones are slower than the estimate says: the CTAs of a wave drift apart and
+// the slabs they share leave the caches.  ENO3 on the default tiles, us per
+// stage by planes per chunk: 81^4 21 431, 27 426, 31 434, 41 474, 81 461; 60^4
+// 10 146, 15 149, 21 166, 41 171; 50 x 90 x 60 x 70 14 206, 23 213, 31 251, 90
+// 258; 30 x 150 x 50 x 64 10 162, 25 158, 31 180, 41 214, 150 308.
 constexpr int kMarchMaxPlanes4 = 28;
 
 // Tiles of the register-marching ENO kernel (stage_march.cuh) for this grid,

@@ -125,9 +125,9 @@ __device__ __forceinline__ bool past_last_step(const StageArgs<R>& a)
 // ordinary loads after it, never through the read-only path, which the wait
 // does not order.  Release comes after the wait: released at the top, several
 // stages queue up on the SMs and a 101 x 101 FP64 stage takes 6.0 us.  Whole
-// solves, ordinary launches -> this: 101 x 101 FP64 graph 540 -> 515 us, 257 x
-// 193 FP32 with device-chosen steps 606 -> 412, air3d 41^3 793 -> 650, car4d
-// 33 x 41 x 37 x 29 549 -> 510, rockets 300^3 1923 -> 1822.
+// solves, ordinary launches -> this: 101 x 101 FP64 graph 515 -> 488 us, 257 x
+// 193 FP32 with device-chosen steps 594 -> 405, air3d 41^3 593 -> 385, car4d
+// 33 x 41 x 37 x 29 551 -> 516, rockets 300^3 1977 -> 1921.
 __device__ __forceinline__ void stage_release()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

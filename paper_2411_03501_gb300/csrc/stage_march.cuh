@@ -31,8 +31,8 @@
 //
 // Measured (GB300, us per stage of whole solves; default tile of the scalar
 // body before, its autotuned tile or run kernel in brackets, this kernel's
-// default tile now): rockets 300^3 ENO2 388 (182), 160; 100^3 20.8 (14.3),
-// 8.5; car4d 81^4 ENO3 870 (650), 438; 33 x 41 x 37 x 29 48, 21.5.  What
+// default tile now): rockets 300^3 ENO2 388 (182), 157; 100^3 20.8 (14.3),
+// 8.9; car4d 81^4 ENO3 870 (650), 425; 33 x 41 x 37 x 29 48, 21.7.  What
 // bounds it: instruction issue (65 % of the cycles on rockets 200^3, 165
 // instructions per node in 3-D and 244 in 4-D, of which 45 and 125 are the
 // scheme's arithmetic) and the latency of the loads between barriers.

@@ -21,10 +21,10 @@ cudaError_t march_launch(const StageArgs<float>& a, const Tile& t, cudaStream_t 
               nchunks * (ND == 4 ? (a.n[0] + R0 - 1) / R0 : 1));
     const size_t smem = 2 * sizeof(float) * R0 * (t.ta + 2 * G) * kMarchPitch;
     const int threads = march_threads(t);
-    // In 4-D a launch of many waves is faster as an ordinary one (car4d 81^4,
-    // 27 planes, 6 waves: 434 us per stage against 503; 33 x 41 x 37 x 29, one
-    // wave: 22.9 against 21.2).  In 3-D the dependent form is faster there too
-    // (rockets 300^3: 160 against 152).
+    // In 4-D a launch of many waves is faster as an ordinary one (us per stage,
+    // ordinary and dependent: car4d 81^4, 27 planes, 6 waves 425, 480; 33 x 41
+    // x 37 x 29, one wave 23.2, 21.7).  In 3-D the dependent form is faster
+    // there too (rockets 300^3 161, 157; 100^3 11.0, 8.9).
     if constexpr (ND == 4) {
         constexpr int kResident = 65536 / 128;  // threads of an SM
         const long long ctas = (long long)grid.x * grid.y * grid.z;

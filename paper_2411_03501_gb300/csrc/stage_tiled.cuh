@@ -107,11 +107,12 @@ __device__ __forceinline__ void deriv_fast(const R* u, R inv_dx, R floor12, R& p
 }
 
 // Loads of the stage input.  COH = false: through the read-only cache (the
-// field does not change during the launch).  COH = true: the persistent
-// batched launch, in which other CTAs of the same launch wrote the field
-// before this CTA's acquire (the fence after it observed their completion
-// count): a weak load cached at every level (ld.global.ca), which that
-// acquire orders, not the read-only path, which no fence orders.
+// field does not change while the kernel's CTAs exist).  COH = true: the field
+// may have been written after the CTA started: by other CTAs of the persistent
+// batched launch before this CTA's acquire (the fence after it observed their
+// completion count), or by the previous stage before stage_wait (kernels of
+// launch_dependent).  A weak load cached at every level (ld.global.ca), which
+// the acquire or the wait orders, not the read-only path, which neither does.
 template <bool COH, typename R>
 __device__ __forceinline__ R ld_in(const R* p)
 {
@@ -139,7 +140,9 @@ struct Tile {
     int minb;        // occupancy target of the kernel variant (2, 3 or 4)
     int pair;        // 0 scalar body; 1 two planes per iteration in paired FP32;
                      // 2 the same with shared WENO5 faces; 3 / 4 face-shared
-                     // ENO runs of 4 / 2 nodes (stage_run.cuh)
+                     // ENO runs of 4 / 2 nodes (stage_run.cuh); 5 both stages
+                     // of an RK2 step (stage_fused.cuh); 6 the marching ENO
+                     // kernel (stage_march.cuh)
 };
 
 // One CTA's share of a stage: the tile (bx, by) of the two fastest axes,
