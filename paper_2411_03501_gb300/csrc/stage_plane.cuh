@@ -51,30 +51,22 @@ __device__ __forceinline__ bool is_finite_bits(double v)
     return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
 }
 
-// 2^k close to 1/e for a normal e > 0: e times it lies in [1, 2).
-__device__ __forceinline__ float near_reciprocal(float e)
+// Power of two that scales q_k = s_k + eps of the WENO5 weights (plane_weno),
+// from eps alone, which is known before the q_k.  Close to 1/eps: then 1 <= q_k
+// <= 4e7, and the products of weights and stencil values reach 3e30 max|v|,
+// which overflows FP32 on rough data from undivided differences of 1e8 on.  In
+// FP32 q_k is therefore scaled 2^13 lower where eps >= 1 (differences from 1e3
+// on): 1.2e-4 <= q_k <= 5e3, products up to 6e14 max|v|, finite up to
+// differences of 1e18.
+__device__ __forceinline__ float weight_scale(float eps)
 {
-    return __uint_as_float(0x7f000000u - (__float_as_uint(e) & 0x7f800000u));
+    const unsigned drop = eps >= 1.0f ? 13u << 23 : 0u;
+    return __uint_as_float(0x7f000000u - (__float_as_uint(eps) & 0x7f800000u) - drop);
 }
-__device__ __forceinline__ double near_reciprocal(double e)
+__device__ __forceinline__ double weight_scale(double eps)
 {
     return __longlong_as_double(0x7fe0000000000000ll -
-                                (__double_as_longlong(e) & 0x7ff0000000000000ll));
-}
-
-// Power of two that scales q_k = s_k + eps of the WENO5 weights (plane_weno).
-// FP32: close to 1/max q_k, so that no product of weights passes 16; scaled by
-// 1/eps (eps <= q_k <= 4e7 eps) their products with the stencil values
-// overflow on rough data from undivided differences of 1e8 on.  FP64 has the
-// range for 1/eps, which is known earlier (max q_k costs 3.7 % of a stage there
-// and 1 % in FP32).
-__device__ __forceinline__ float weight_scale(float, float q1, float q2, float q3)
-{
-    return near_reciprocal(fmaxf(fmaxf(q1, q2), q3));
-}
-__device__ __forceinline__ double weight_scale(double eps, double, double, double)
-{
-    return near_reciprocal(eps);
+                                (__double_as_longlong(eps) & 0x7ff0000000000000ll));
 }
 
 // weno5_combine (stencil.cuh) with one division instead of four: the weights
@@ -96,9 +88,8 @@ __device__ __forceinline__ R plane_weno(R v1, R v2, R v3, R v4, R v5, R floor_)
     const R s3 = R(13.0 / 12.0) * a3 * a3 + R(0.25) * b3 * b3;
     const R m = mag_max(mag_max(mag_max(v1, v2), mag_max(v3, v4)), v5);
     const R eps = R(1e-6) * (m * m) + floor_;
-    const R t1 = s1 + eps, t2 = s2 + eps, t3 = s3 + eps;
-    const R sc = weight_scale(eps, t1, t2, t3);
-    const R q1 = t1 * sc, q2 = t2 * sc, q3 = t3 * sc;
+    const R sc = weight_scale(eps);
+    const R q1 = (s1 + eps) * sc, q2 = (s2 + eps) * sc, q3 = (s3 + eps) * sc;
     const R Q1 = q1 * q1, Q2 = q2 * q2, Q3 = q3 * q3;
     const R al1 = R(0.1) * (Q2 * Q3), al2 = R(0.6) * (Q1 * Q3), al3 = R(0.3) * (Q1 * Q2);
     return (al1 * phi1 + al2 * phi2 + al3 * phi3) / (al1 + al2 + al3);
