@@ -22,7 +22,7 @@ static cudaError_t plane_dyn(int dyn, const StageArgs<LSP_REAL>& a, cudaStream_t
     const int nt = plane_block(a.npts, sm_count());
     int nb = (a.npts + nt - 1) / nt;
     if (sizeof(LSP_REAL) == 8) nb = std::min(nb, 16 * sm_count());
-    const PlaneConst<LSP_REAL> pc = plane_const(a);
+    const PlaneConst<LSP_REAL> pc(a);
     switch (dyn) {
     case NORMAL_SPEED: return launch_dependent(stage_plane_kernel<SCHEME, NORMAL_SPEED, LSP_REAL>, nb, nt, 0, s, a, pc);
     case TRANSLATE: return launch_dependent(stage_plane_kernel<SCHEME, TRANSLATE, LSP_REAL>, nb, nt, 0, s, a, pc);
@@ -94,7 +94,7 @@ static cudaError_t prange_plane(int scheme, const StageArgs<LSP_REAL>& a, const 
                                 cudaStream_t s)
 {
     const int nt = plane_block(a.npts, sm_count()), nb = (a.npts + nt - 1) / nt;
-    const PlaneConst<LSP_REAL> pc = plane_const(a);
+    const PlaneConst<LSP_REAL> pc(a);
     switch (scheme) {
     case UPWIND1: return launch_dependent(prange_plane_kernel<UPWIND1, LSP_REAL>, nb, nt, 0, s, a, pc, ch);
     case ENO2: return launch_dependent(prange_plane_kernel<ENO2, LSP_REAL>, nb, nt, 0, s, a, pc, ch);

@@ -142,27 +142,53 @@ __device__ __forceinline__ void plane_window(const R* p, int c, int n, int s,
     if (!inside && !periodic) fix_extrapolated<1, G>(u, c, n);
 }
 
-// Constants of a launch, formed on the host: a thread has few nodes, and what
-// it forms once costs FP64 operations (101 x 101 FP64 ENO2 4.6 -> 4.4 us per
-// stage of a graph; 2048^2 FP64 first order 282 -> 264).
+// Constants of a launch.  FP64: formed on the host, since a thread has few
+// nodes and what it forms once costs FP64 operations (101 x 101 FP64 ENO2 4.6
+// -> 4.4 us per stage of a graph; 2048^2 FP64 first order 282 -> 264).  FP32:
+// formed by each thread, 1 to 2 % faster than loading them (4096^2 ENO3 162.3,
+// 160.1 us).
 template <typename R>
-struct PlaneConst {
-    R cl;         // c_l dt (dt not from the control block)
-    R half[2];    // alpha / 2 (alpha not from the control block)
-    R floor_[2];  // floor of WENO5's epsilon
+struct PlaneConst;
+
+template <>
+struct PlaneConst<float> {
+    explicit PlaneConst(const StageArgs<float>&) {}
+    __device__ __forceinline__ float rate_factor(const StageArgs<float>& a) const  // c_l dt
+    {
+        return a.c_l * (a.dt_from_ctl ? float(a.ctl->dt) : a.dt);
+    }
+    __device__ __forceinline__ float half_alpha(const StageArgs<float>& a, int k) const
+    {
+        return (a.alpha_from_ctl ? float(__longlong_as_double((long long)a.ctl->alpha_bits[k])) : a.alpha[k]) *
+               0.5f;
+    }
+    __device__ __forceinline__ float floor_(const StageArgs<float>& a, int k) const
+    {
+        return Num<float>::eps_floor(a.inv_dx[k]);
+    }
 };
 
-template <typename R>
-PlaneConst<R> plane_const(const StageArgs<R>& a)
-{
-    PlaneConst<R> p;
-    p.cl = a.c_l * a.dt;
-    for (int k = 0; k < 2; ++k) {
-        p.half[k] = a.alpha[k] * R(0.5);
-        p.floor_[k] = Num<R>::eps_floor(a.inv_dx[k]);
+template <>
+struct PlaneConst<double> {
+    double cl, half[2], fl[2];
+    explicit PlaneConst(const StageArgs<double>& a)
+    {
+        cl = a.c_l * a.dt;
+        for (int k = 0; k < 2; ++k) {
+            half[k] = a.alpha[k] * 0.5;
+            fl[k] = Num<double>::eps_floor(a.inv_dx[k]);
+        }
     }
-    return p;
-}
+    __device__ __forceinline__ double rate_factor(const StageArgs<double>& a) const
+    {
+        return a.dt_from_ctl ? a.c_l * a.ctl->dt : cl;
+    }
+    __device__ __forceinline__ double half_alpha(const StageArgs<double>& a, int k) const
+    {
+        return a.alpha_from_ctl ? __longlong_as_double((long long)a.ctl->alpha_bits[k]) * 0.5 : half[k];
+    }
+    __device__ __forceinline__ double floor_(const StageArgs<double>&, int k) const { return fl[k]; }
+};
 
 // A thread takes one node (FP32) or the nodes of a grid-stride loop (FP64, at
 // most 16 blocks per SM: 4096^2 first order 1038 us in one pass of blocks,
@@ -182,17 +208,16 @@ __global__ void __launch_bounds__(256) stage_plane_kernel(StageArgs<R> a, PlaneC
         plane_window<G>(a.phi_s + idx, j, a.n[1], 1, a.periodic[1], u[1]);
         const R vn = a.phi_n ? a.phi_n[idx] : R(0);
         const R g = a.tube ? a.target[idx] : R(0);
-        const R cl = a.dt_from_ctl ? a.c_l * R(a.ctl->dt) : pc.cl;
+        const R cl = pc.rate_factor(a);
         const R x[2] = {rfma(R(i), a.h[0], a.lo[0]), rfma(R(j), a.h[1], a.lo[1])};
         R pbar[2], diss = R(0);
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             R pm, pp;
-            plane_derivs<SCHEME>(u[k], pc.floor_[k], pm, pp);
+            plane_derivs<SCHEME>(u[k], pc.floor_(a, k), pm, pp);
             pm *= a.inv_dx[k];
             pp *= a.inv_dx[k];
-            R ha = pc.half[k];  // alpha / 2
-            if (a.alpha_from_ctl) ha = R(__longlong_as_double((long long)a.ctl->alpha_bits[k])) * R(0.5);
+            R ha = pc.half_alpha(a, k);
             if (a.local_alpha) ha = local_alpha<DYN>(x, k, a.prm, R(0), R(1), pm, pp) * R(0.5);
             pbar[k] = R(0.5) * (pp + pm);
             diss += ha * (pp - pm);
@@ -231,7 +256,7 @@ __global__ void __launch_bounds__(256) prange_plane_kernel(StageArgs<R> a, Plane
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             R am, ap;
-            plane_derivs<SCHEME>(u[k], pc.floor_[k], am, ap);
+            plane_derivs<SCHEME>(u[k], pc.floor_(a, k), am, ap);
             m[k] = rmax(rabs(am), rabs(ap)) * a.inv_dx[k];
         }
     }
