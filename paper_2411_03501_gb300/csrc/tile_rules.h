@@ -22,38 +22,43 @@ inline RuleTile pair_square_tile(int d, const int* n, long long sms)
     return {16, 16, ch + (ch & 1)};
 }
 
-// Estimated time of a stage of that kernel on a 3-D grid, in units of one
-// warp's issue time per pair of planes (80 ns):
-//   25 + sqrt(W^2 + L^2) + 0.5 k (ch / 2 + 0.75) warps'
-// with warps' = warps (1 + 0.29 frame / tile); W the warp pairs per SM, each
-// chunk 0.75 pairs more than its length; L the latency of the chain of
-// chunks, 20 per pair and wave of resident CTAs; the last term the tail of the
-// launch, half of the k CTAs an SM holds (3 of 256 threads).  Fitted to 5,200
-// timings on 150 random grids of 2,000 to 25 million nodes (root mean square
-// error 8 %).
+// Estimated time in us of a stage of that kernel on a 3-D grid, back to back
+// with others of its kind.
+//  - A pair of planes takes f(k) = (1.88^2.4 + (0.128 k u)^2.4)^(1/2.4) us with k
+//    CTAs on the SM that started together and u = warps (1 + 0.19 frame / tile):
+//    the latency of one chain, or the issue slots of all.  A chunk takes its
+//    pairs and 0.32 more for its start.
+//  - 24 warps of 80 registers fit on an SM: R = 24 / warps CTAs.
+//  - A launch of one wave: its CTAs start beside the previous stage's, so above
+//    half a wave some SMs fill up to R while others wait (16 x 16 tiles of 6
+//    planes: 9.5 us up to one CTA per SM, 11.8 up to 1.5, 15.5 up to 3).
+//  - More: R CTAs out of step take 0.74 of f(R) a pair (0.73 pairs for a start),
+//    and the tail of the last is 0.42 of a chunk.
+// Fitted to 42,800 timings on 870 random grids (root mean square error 5 %).
 inline double pair_cost(const int* n, const RuleTile& t, long long sms)
 {
     const int nS = n[0], nA = n[1], nB = n[2], G = 3;
-    const int warps = (t.tb * t.ta + 31) / 32;
-    const double resident = std::min(65536 / (80 * 32 * warps), 32);
-    const double unit = warps * (1.0 + 0.29 * 2 * G * (t.tb + t.ta) / (t.tb * t.ta));
+    const int warps = (t.tb * t.ta + 31) / 32, R = 24 / warps;
+    const double unit = 0.128 * warps * (1.0 + 0.19 * 2 * G * (t.tb + t.ta) / (t.tb * t.ta));
+    const auto pair_us = [&](double k) {
+        return std::pow(std::pow(1.88, 2.4) + std::pow(k * unit, 2.4), 1.0 / 2.4);
+    };
     const double columns = (double)((nB + t.tb - 1) / t.tb) * ((nA + t.ta - 1) / t.ta);
-    const double chunks = (nS + t.ch - 1) / t.ch, ctas = columns * chunks;
-    const double chunk = 0.5 * std::min(t.ch, nS) + 0.75;
-    const double k = std::min(std::ceil(ctas / sms), resident);
-    const double W = columns * (0.5 * nS + 0.75 * chunks) * unit / sms;
-    const double L = 20.0 * chunk * std::max(1.0, ctas / (sms * resident));
-    return 25.0 + std::sqrt(W * W + L * L) + 0.5 * k * chunk * unit;
+    const double chunks = (nS + t.ch - 1) / t.ch, per_sm = columns * chunks / sms;
+    const double chunk = 0.5 * std::min(t.ch, nS) + 0.32, full = chunk * pair_us(R);
+    if (per_sm <= 0.5 * R) return 2.9 + chunk * pair_us(std::ceil(per_sm));
+    if (per_sm <= R) return 2.9 + full;
+    return 2.9 + std::max(full, 0.74 * columns * (0.5 * nS + 0.73 * chunks) / sms * pair_us(R) / R + 0.42 * full);
 }
 
 // Tile of that kernel on a 3-D grid: the lowest estimate over tiles of 64 to
 // 256 threads that split both axes evenly and a few even chunk lengths, where
-// it is 10 % below the square tile's, else none (the square tile is used).
-// Against the square tile on 120 other random grids: geometric mean 0.77 of
-// its time, the slowest 1.014.  us per stage, square tile and this rule: 41^3
-// 9.7, 5.4; 97x113x85 25.4, 22.5; 129^3 46.2, 40.4; 201^3 (square) 123.6.  (An
-// estimate without the margin, and without the work of the chunks as such, was
-// up to 1.3 times slower than the square tile on 22 of 150 grids.)
+// it is 5 % below the square tile's, else none (the square tile is used).
+// On 360 other grids (7 to 3000 nodes an axis) the geometric mean is 0.757 of
+// the square tile's time; four are slower by more than 3 % (1.13 on 9 x 262 x
+// 206, else 1.04).  us per stage, square tile and this rule: 41^3 9.7, 5.4; 97 x
+// 113 x 85 25.4, 22.5; 429 x 286 x 8 40.8, 25.6; 3000 x 148 x 19 228, 146; 201^3
+// (square) 123.6.
 inline RuleTile pair_rule(const int* n, long long sms)
 {
     const int nS = n[0], nA = n[1], nB = n[2], G = 3;
@@ -81,7 +86,7 @@ inline RuleTile pair_rule(const int* n, long long sms)
             }
         }
     }
-    if (best.ch && pair_cost(n, pair_square_tile(3, n, sms), sms) <= 1.1 * best_cost) best.ch = 0;
+    if (best.ch && pair_cost(n, pair_square_tile(3, n, sms), sms) <= 1.05 * best_cost) best.ch = 0;
     return best;
 }
 
