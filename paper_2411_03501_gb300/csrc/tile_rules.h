@@ -35,21 +35,32 @@ inline RuleTile pair_square_tile(int d, const int* n, long long sms)
 //  - More: R CTAs out of step take 0.74 of f(R) a pair (0.73 pairs for a start),
 //    and the tail of the last is 0.42 of a chunk.
 // Fitted to 42,800 timings on 870 random grids (root mean square error 5 %).
-inline double pair_cost(const int* n, const RuleTile& t, long long sms)
-{
-    const int nS = n[0], nA = n[1], nB = n[2], G = 3;
-    const int warps = (t.tb * t.ta + 31) / 32, R = 24 / warps;
-    const double unit = 0.128 * warps * (1.0 + 0.19 * 2 * G * (t.tb + t.ta) / (t.tb * t.ta));
-    const auto pair_us = [&](double k) {
-        return std::pow(std::pow(1.88, 2.4) + std::pow(k * unit, 2.4), 1.0 / 2.4);
-    };
-    const double columns = (double)((nB + t.tb - 1) / t.tb) * ((nA + t.ta - 1) / t.ta);
-    const double chunks = (nS + t.ch - 1) / t.ch, per_sm = columns * chunks / sms;
-    const double chunk = 0.5 * std::min(t.ch, nS) + 0.32, full = chunk * pair_us(R);
-    if (per_sm <= 0.5 * R) return 2.9 + chunk * pair_us(std::ceil(per_sm));
-    if (per_sm <= R) return 2.9 + full;
-    return 2.9 + std::max(full, 0.74 * columns * (0.5 * nS + 0.73 * chunks) / sms * pair_us(R) / R + 0.42 * full);
-}
+struct PairCost {
+    int nS, R;
+    double unit, columns, sms, full_pair;
+    PairCost(const int* n, int tb, int ta, long long sms_)
+    {
+        const int nA = n[1], nB = n[2], G = 3, warps = (tb * ta + 31) / 32;
+        nS = n[0];
+        R = 24 / warps;
+        unit = 0.128 * warps * (1.0 + 0.19 * 2 * G * (tb + ta) / (tb * ta));
+        columns = (double)((nB + tb - 1) / tb) * ((nA + ta - 1) / ta);
+        sms = (double)sms_;
+        full_pair = pair_us(R);
+    }
+    double pair_us(double k) const
+    {
+        return std::pow(4.5498 + std::pow(k * unit, 2.4), 1.0 / 2.4);  // 1.88^2.4
+    }
+    double operator()(int ch) const
+    {
+        const double chunks = (nS + ch - 1) / ch, per_sm = columns * chunks / sms;
+        const double chunk = 0.5 * std::min(ch, nS) + 0.32, full = chunk * full_pair;
+        if (per_sm <= 0.5 * R) return 2.9 + chunk * pair_us(std::ceil(per_sm));
+        if (per_sm <= R) return 2.9 + full;
+        return 2.9 + std::max(full, 0.74 * columns * (0.5 * nS + 0.73 * chunks) / sms * full_pair / R + 0.42 * full);
+    }
+};
 
 // Tile of that kernel on a 3-D grid: the lowest estimate over tiles of 64 to
 // 256 threads that split both axes evenly and a few even chunk lengths, where
@@ -74,19 +85,20 @@ inline RuleTile pair_rule(const int* n, long long sms)
             if (!even(nA, ta) || (nA + ta - 1) / ta > 65535) continue;
             // the haloed tile in 3 values per thread
             if ((ta + 2 * G) * (tb + 2 * G) > 3 * ta * tb) continue;
+            const PairCost cost(n, tb, ta, sms);
             for (const int ch : {2, 4, 6, 8, 10, 12, 16, 20, 26, 34, 50, 66, 102}) {
                 if (ch > nS + 1) break;
-                const RuleTile t{tb, ta, ch};
                 if ((nS + ch - 1) / ch > 65535) continue;
-                const double c = pair_cost(n, t, sms);
+                const double c = cost(ch);
                 if (best.ch == 0 || c < best_cost) {
-                    best = t;
+                    best = {tb, ta, ch};
                     best_cost = c;
                 }
             }
         }
     }
-    if (best.ch && pair_cost(n, pair_square_tile(3, n, sms), sms) <= 1.05 * best_cost) best.ch = 0;
+    const RuleTile square = pair_square_tile(3, n, sms);
+    if (best.ch && PairCost(n, square.tb, square.ta, sms)(square.ch) <= 1.05 * best_cost) best.ch = 0;
     return best;
 }
 
