@@ -119,7 +119,8 @@ typedef struct {
                           one graph and launches that                      */
     int batch_chunk;   /* batched solves: planes per CTA along the march of
                           3-D/4-D problems (0 = 4 to 128 by the work per
-                          resident CTA of one stage of the batch)         */
+                          resident CTA of one stage of the batch, whole
+                          columns where they fill the device)             */
     int batch_persistent; /* batched solves: 1 = the whole solve as ONE
                           launch of resident CTAs that take (step, stage,
                           tile) items in order and wait on per-problem
@@ -347,7 +348,7 @@ lsp_status lsp_hj_solve_noalloc(lsp_grid* grid, const lsp_solve_opts* opts, void
  * problem dimension at a time (coordinate descent from opts->batch_tiles),
  * and returns the fastest in *batch_tiles for the caller to store in
  * opts->batch_tiles.  Arguments as for lsp_hj_solve_batched; the workspace
- * from lsp_batched_workspace_size serves every tile choice.  Waits for the
+ * from lsp_batched_workspace_size serves every tile choice and both forms.  Waits for the
  * GPU. */
 lsp_status lsp_batched_autotune(int nprob, lsp_grid* const* grids, const lsp_solve_opts* opts,
                                 const void* const* phis, const void* const* targets,
