@@ -36,7 +36,8 @@ def shim(tmp_path_factory):
         os.path.realpath(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc")))
     d = tmp_path_factory.mktemp("smem")
     (d / "shim.cpp").write_text(SHIM)
-    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-I", cuda + "/include",
+    # its own stand-in, whatever runtime the process has loaded
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", CSRC, "-I", cuda + "/include",
                     str(d / "shim.cpp"), "-o", str(d / "shim.so")], check=True)
     return ctypes.CDLL(str(d / "shim.so"))
 
